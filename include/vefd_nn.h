@@ -64,6 +64,24 @@ int vefd_nn_pack_weights(const float *w, int Cout, int K27, int Kp, void *wb, vo
 /* dw[o][k] (+)= sum_s parts[s][k][o] for k < K27 (parts: split-K slices of dW^T, stride split_stride). */
 int vefd_nn_splitk_reduce_t(const float *parts, int splits, long long split_stride, int Kp, int Cout, int K27,
                             float *dw, int accumulate, void *stream);
+/* The same layers without the im2col matrix: the products gather 16-byte
+ * pieces (8 channels) of a BF16 copy of the activations, xb[voxel][8 C8], C8 =
+ * ceil(Cin / 8), zero padded.  Cout a multiple of 8; xb, wk, wd, y, dy and
+ * scratch 16-byte aligned.
+ * conv3d_sizes: BF16 elements of the two packed weight arrays of a layer. */
+void vefd_nn_conv3d_sizes(int Cin, int Cout, long long *wk, long long *wd);
+/* w[Cout][27 Cin] -> wk (forward) and wd (backward data), BF16 (layouts in nn_conv.cu). */
+int vefd_nn_conv3d_pack(const float *w, int Cin, int Cout, void *wk, void *wd, void *stream);
+/* y[v'][o] = act(sum + bias[o]) (bias may be NULL; act max(., 0) when relu); writes xb for the backward pass. */
+int vefd_nn_conv3d_forward(const float *x, int B, int D, int H, int W, int Cin, int stride, const void *wk,
+                           const float *bias, int Cout, int relu, void *xb, float *y, unsigned *status, void *stream);
+/* Floats of scratch the backward pass needs (0 for bad sizes). */
+long long vefd_nn_conv3d_backward_scratch(int B, int D, int H, int W, int Cin, int stride, int Cout);
+/* Gradients for the output gradient dy: dw[o][k] and db[o] (added when accumulate), dx (overwritten); y the
+ * forward output (its sign masks dy when relu).  The output voxels must be a multiple of 8. */
+int vefd_nn_conv3d_backward(const void *xb, const float *y, const float *dy, int B, int D, int H, int W, int Cin,
+                            int stride, const void *wd, int Cout, int relu, float *scratch, float *dw, float *db,
+                            int accumulate, float *dx, unsigned *status, void *stream);
 /* Nearest-neighbour upsampling by 2 of x [B][D][H][W][C] and its adjoint (sum of the 8 children). */
 int vefd_nn_upsample2(const float *x, int B, int D, int H, int W, int C, float *y, void *stream);
 int vefd_nn_upsample2_backward(const float *dy, int B, int D, int H, int W, int C, float *dx, int accumulate,

@@ -25,53 +25,13 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "nn_tc.cuh"
 #include "vefd_nn.h"
 
 namespace vefd_nn {
 namespace {
 
 constexpr int kBM = 128, kBK = 64, kThreads = 128;
-constexpr unsigned kStatusTimeout = 1u;
-
-__device__ __forceinline__ unsigned smem_addr(const void* p) {
-    return static_cast<unsigned>(__cvta_generic_to_shared(p));
-}
-
-// Shared-memory matrix descriptor (no swizzle): start address, leading
-// (between core matrices along K) and stride (between 8-row groups) byte
-// offsets, all in 16-byte units, descriptor version 1.
-__device__ __forceinline__ uint64_t smem_desc(unsigned addr, unsigned lbo, unsigned sbo) {
-    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
-// Instruction descriptor of kind::f16: FP32 accumulator, BF16 A and B, both
-// K-major, N >> 3 and M >> 4 in their fields.
-__host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-
-__device__ __forceinline__ void mbar_init1(unsigned bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-// Bounded wait for the phase with the given parity: at most 2^31 SM cycles
-// of clock64 (about one second at 2.07 GHz) and 2^22 polls.
-__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
-    const long long t0 = clock64();
-    for (int it = 0; it < (1 << 22); ++it) {
-        unsigned done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
-        if (clock64() - t0 > (1LL << 31)) break;
-    }
-    return false;
-}
 
 // Byte offset of element (r, k) of a rows x 64 K-major tile in the core-matrix
 // layout: core matrix (r / 8, k / 8) at (r / 8) * sbo + (k / 8) * lbo, its row

@@ -75,6 +75,9 @@ _MORE = {
     "vefd_nn_colsum": "vp ll i vp vp i vp",
     "vefd_nn_pack_weights": "vp i i i vp vp vp",
     "vefd_nn_splitk_reduce_t": "vp i ll i i i vp i vp",
+    "vefd_nn_conv3d_pack": "vp i i vp vp vp",
+    "vefd_nn_conv3d_forward": "vp i i i i i i vp vp i i vp vp vp vp",
+    "vefd_nn_conv3d_backward": "vp vp vp i i i i i i vp i i vp vp vp i vp vp vp",
     "vefd_nn_upsample2": "vp i i i i i vp vp",
     "vefd_nn_upsample2_backward": "vp i i i i i vp i vp",
     "vefd_nn_concat": "vp i vp i ll vp vp",
@@ -85,7 +88,7 @@ _MORE = {
     "vefd_nn_to_fields": "vp vp ll f f f f vp vp vp vp vp",
     "vefd_nn_scale": "vp ll f vp",
 }
-NN_EXPORTS += list(_MORE) + ["vefd_nn_colsum_scratch"]
+NN_EXPORTS += list(_MORE) + ["vefd_nn_colsum_scratch", "vefd_nn_conv3d_sizes", "vefd_nn_conv3d_backward_scratch"]
 _more_done = False
 
 
@@ -100,6 +103,11 @@ def L():
             fn.restype = ctypes.c_int
         lb.vefd_nn_colsum_scratch.argtypes = [ctypes.c_longlong, ctypes.c_int]
         lb.vefd_nn_colsum_scratch.restype = ctypes.c_longlong
+        pll = ctypes.POINTER(ctypes.c_longlong)
+        lb.vefd_nn_conv3d_sizes.argtypes = [ctypes.c_int, ctypes.c_int, pll, pll]
+        lb.vefd_nn_conv3d_sizes.restype = None
+        lb.vefd_nn_conv3d_backward_scratch.argtypes = [ctypes.c_int] * 7
+        lb.vefd_nn_conv3d_backward_scratch.restype = ctypes.c_longlong
         _more_done = True
     return lb
 
@@ -114,16 +122,16 @@ def round8(n):
 
 class Conv3d:
     """3x3x3 convolution, zero padding 1, stride 1 or 2, on channels-last FP32
-    activations [B, D, H, W, C]: im2col, tensor-core GEMM, bias, optional ReLU.
-    FP32 master weights w [Cout, 27 Cin] (tap-major columns), BF16 copies for
-    the products, Adam moments."""
+    activations [B, D, H, W, C], with bias and optional ReLU: implicit GEMMs on
+    the tensor cores over a BF16 copy of the activations (no im2col matrix).
+    FP32 master weights w [Cout, 27 Cin] (tap-major columns), packed BF16
+    copies for the products (pack() after w has changed), Adam moments."""
 
     def __init__(self, cin, cout, stride=1, relu=True, gen=None):
         import torch
         assert cout % 8 == 0 and stride in (1, 2)
         self.cin, self.cout, self.stride, self.relu = cin, cout, stride, relu
         self.K27 = 27 * cin
-        self.Kp = round8(self.K27)
         std = (2.0 / self.K27) ** 0.5
         w = torch.randn(cout, self.K27, generator=gen) * std
         self.w = w.cuda()
@@ -132,8 +140,10 @@ class Conv3d:
         self.db = torch.zeros_like(self.b)
         self.mw, self.vw = torch.zeros_like(self.w), torch.zeros_like(self.w)
         self.mb, self.vb = torch.zeros_like(self.b), torch.zeros_like(self.b)
-        self.wb = torch.empty(cout, self.Kp, dtype=torch.bfloat16, device="cuda")
-        self.wbT = torch.empty(self.Kp, cout, dtype=torch.bfloat16, device="cuda")
+        nk, nd = ctypes.c_longlong(), ctypes.c_longlong()
+        L().vefd_nn_conv3d_sizes(cin, cout, ctypes.byref(nk), ctypes.byref(nd))
+        self.wk = torch.empty(nk.value, dtype=torch.bfloat16, device="cuda")
+        self.wd = torch.empty(nd.value, dtype=torch.bfloat16, device="cuda")
         self.status = torch.zeros(1, dtype=torch.int32, device="cuda")
         self.pack()
 
@@ -141,8 +151,8 @@ class Conv3d:
         return [(self.w, self.dw, self.mw, self.vw), (self.b, self.db, self.mb, self.vb)]
 
     def pack(self):
-        _check(L().vefd_nn_pack_weights(_p(self.w), self.cout, self.K27, self.Kp, _p(self.wb), _p(self.wbT),
-                                        _stream()), "pack_weights")
+        _check(L().vefd_nn_conv3d_pack(_p(self.w), self.cin, self.cout, _p(self.wk), _p(self.wd), _stream()),
+               "conv3d_pack")
 
     def out_shape(self, shape):
         B, D, H, W, _ = shape
@@ -153,45 +163,27 @@ class Conv3d:
         import torch
         B, D, H, W, C = x.shape
         assert C == self.cin and x.is_contiguous()
-        oshape = self.out_shape(x.shape)
-        V = oshape[0] * oshape[1] * oshape[2] * oshape[3]
-        col = torch.empty(V, self.Kp, dtype=torch.bfloat16, device="cuda")
-        colT = torch.empty(self.Kp, V, dtype=torch.bfloat16, device="cuda")
-        _check(L().vefd_nn_im2col3d(_p(x), B, D, H, W, C, self.stride, self.Kp, _p(col), _p(colT), _stream()),
-               "im2col")
-        y = torch.empty(V, self.cout, dtype=torch.float32, device="cuda")
-        gemm(col, self.wb, C=y, status=self.status)
-        _check(L().vefd_nn_bias_act(_p(y), _p(self.b), V, self.cout, int(self.relu), _stream()), "bias_act")
-        self._saved = (x.shape, colT, y)
-        return y.view(oshape)
+        y = torch.empty(self.out_shape(x.shape), device="cuda")
+        xb = torch.empty(B * D * H * W, round8(C), dtype=torch.bfloat16, device="cuda")
+        _check(L().vefd_nn_conv3d_forward(_p(x), B, D, H, W, C, self.stride, _p(self.wk), _p(self.b), self.cout,
+                                          int(self.relu), _p(xb), _p(y), _p(self.status), _stream()), "conv3d_forward")
+        self._saved = (x.shape, xb, y)
+        return y
 
     def backward(self, dy, accumulate=False):
         """Gradients of w and b (added when accumulate) and of the input."""
         import torch
-        xshape, colT, y = self._saved
+        xshape, xb, y = self._saved
         B, D, H, W, C = xshape
-        V = y.shape[0]
-        dy = dy.reshape(V, self.cout).contiguous()
-        g = torch.empty_like(y)
-        gb = torch.empty(V, self.cout, dtype=torch.bfloat16, device="cuda")
-        gbT = torch.empty(self.cout, V, dtype=torch.bfloat16, device="cuda")
-        lb, s = L(), _stream()
-        _check(lb.vefd_nn_act_backward(_p(dy), _p(y), V, self.cout, int(self.relu), _p(g), _p(gb), _p(gbT), s),
-               "act_backward")
-        scratch = torch.empty(lb.vefd_nn_colsum_scratch(V, self.cout), device="cuda")
-        _check(lb.vefd_nn_colsum(_p(g), V, self.cout, _p(scratch), _p(self.db), int(accumulate), s), "colsum")
-        # dW^T [Kp, Cout] = col^T [Kp, V] . g [V, Cout], split over the voxels
-        ksplit = max(64, ((V + 63) // 64 + 127) // 128 * 64)
-        splits = (V + ksplit - 1) // ksplit
-        parts = torch.empty(splits, self.Kp, self.cout, device="cuda")
-        _check(lb.vefd_nn_gemm_bf16_splitk(_p(colT), V, _p(gbT), V, _p(parts), self.cout, self.Kp, self.cout, V,
-                                           ksplit, self.Kp * self.cout, _p(self.status), s), "gemm_splitk")
-        _check(lb.vefd_nn_splitk_reduce_t(_p(parts), splits, self.Kp * self.cout, self.Kp, self.cout, self.K27,
-                                          _p(self.dw), int(accumulate), s), "splitk_reduce")
-        # dcol [V, Kp] = g [V, Cout] . W [Cout, Kp]; col2im onto the input
-        dcol = gemm(gb, self.wbT, status=self.status)
-        dx = torch.empty(B, D, H, W, C, device="cuda")
-        _check(lb.vefd_nn_col2im3d(_p(dcol), B, D, H, W, C, self.stride, self.Kp, _p(dx), s), "col2im")
+        dy = dy.reshape(y.shape).contiguous()
+        if dy.data_ptr() % 16:
+            dy = dy.clone()
+        lb, size = L(), (B, D, H, W, C, self.stride)
+        scratch = torch.empty(lb.vefd_nn_conv3d_backward_scratch(*size, self.cout), device="cuda")
+        dx = torch.empty(xshape, device="cuda")
+        _check(lb.vefd_nn_conv3d_backward(_p(xb), _p(y), _p(dy), *size, _p(self.wd), self.cout, int(self.relu),
+                                          _p(scratch), _p(self.dw), _p(self.db), int(accumulate), _p(dx),
+                                          _p(self.status), _stream()), "conv3d_backward")
         self._saved = None
         return dx
 

@@ -159,6 +159,38 @@ def test_conv_layer_matches_torch(cin, cout, stride, relu, shape):
     assert int(lay.status.item()) == 0
 
 
+@pytest.mark.parametrize("cin,cout,stride,shape", [
+    (8, 8, 1, (1, 1, 1, 8)), (8, 16, 2, (1, 5, 3, 16)), (3, 24, 1, (2, 3, 5, 8)), (24, 40, 1, (1, 7, 9, 8)),
+    (48, 16, 1, (1, 6, 10, 24)), (16, 264, 1, (1, 2, 3, 8)), (232, 80, 1, (1, 4, 4, 8)), (40, 152, 2, (2, 7, 6, 16)),
+    (16, 32, 2, (1, 2, 1, 16)), (64, 256, 1, (1, 3, 3, 8))])
+def test_conv_gather_products(cin, cout, stride, shape):
+    """The gathered products at the edges of their tiles (one voxel row, ragged
+    rows and channel slabs, several column tiles, odd sizes at stride 2) against
+    FP64 of the BF16 operands they multiply: only FP32 accumulation is left,
+    over K terms an error below sqrt(K) 2^-23 of the terms' size; 1e-5 sqrt(K)
+    of the largest value is the bound of the other products here."""
+    import torch
+    import torch.nn.functional as F
+    from paper_1406_2686_gb300 import nn
+    g = torch.Generator().manual_seed(cin * 7 + cout)
+    lay = nn.Conv3d(cin, cout, stride, False, gen=g)
+    x = torch.randn(*shape, cin, generator=g)
+    y = lay.forward(x.cuda().contiguous())
+    dy = torch.randn(*y.shape, generator=g).to(torch.bfloat16).float()
+    dx = lay.backward(dy.cuda())
+    torch.cuda.synchronize()
+    assert int(lay.status.item()) == 0
+    xr = _ncdhw(x.to(torch.bfloat16).double()).requires_grad_(True)
+    wr = _torch_weight(lay).requires_grad_(True)
+    yr = F.conv3d(xr, wr, None, stride=stride, padding=1)
+    yr.backward(_ncdhw(dy.double()))
+    V = y.numel() // cout
+    for got, ref, K in ((_ncdhw(y.cpu().double()), yr.detach(), 27 * cin), (_ncdhw(dx.cpu().double()), xr.grad, 27 * cout),
+                        (lay.dw.cpu().double(), wr.grad.permute(0, 2, 3, 4, 1).reshape(cout, -1), V),
+                        (lay.db.cpu().double(), dy.double().sum((0, 1, 2, 3)), V)):
+        assert float((got - ref).abs().max()) < _tol(ref, K)
+
+
 @pytest.mark.parametrize("channels", [(8, 16, 32, 64), (8, 16, 24, 40)])
 def test_unet_gradients_match_torch(channels):
     """The whole U-Net (forward, MSE loss, backward through every layer, skip
