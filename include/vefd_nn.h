@@ -64,14 +64,14 @@ int vefd_nn_pack_weights(const float *w, int Cout, int K27, int Kp, void *wb, vo
 /* dw[o][k] (+)= sum_s parts[s][k][o] for k < K27 (parts: split-K slices of dW^T, stride split_stride). */
 int vefd_nn_splitk_reduce_t(const float *parts, int splits, long long split_stride, int Kp, int Cout, int K27,
                             float *dw, int accumulate, void *stream);
-/* The same layers without the im2col matrix: the products gather 16-byte
+/* The same layers without the im2col matrix: the products read 16-byte
  * pieces (8 channels) of a BF16 copy of the activations, xb[voxel][8 C8], C8 =
  * ceil(Cin / 8), zero padded.  Cout a multiple of 8; xb, wk, wd, y, dy and
  * scratch 16-byte aligned.
  * conv3d_sizes: BF16 elements of the two packed weight arrays of a layer. */
-void vefd_nn_conv3d_sizes(int Cin, int Cout, long long *wk, long long *wd);
+int vefd_nn_conv3d_sizes(int Cin, int Cout, int stride, long long *wk, long long *wd);
 /* w[Cout][27 Cin] -> wk (forward) and wd (backward data), BF16 (layouts in nn_conv.cu). */
-int vefd_nn_conv3d_pack(const float *w, int Cin, int Cout, void *wk, void *wd, void *stream);
+int vefd_nn_conv3d_pack(const float *w, int Cin, int Cout, int stride, void *wk, void *wd, void *stream);
 /* y[v'][o] = act(sum + bias[o]) (bias may be NULL; act max(., 0) when relu); writes xb for the backward pass. */
 int vefd_nn_conv3d_forward(const float *x, int B, int D, int H, int W, int Cin, int stride, const void *wk,
                            const float *bias, int Cout, int relu, void *xb, float *y, unsigned *status, void *stream);

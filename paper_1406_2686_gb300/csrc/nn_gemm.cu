@@ -423,23 +423,11 @@ int launch_gemm(const void* A, int lda, const void* B, int ldb, float* C, int ld
 }  // namespace
 
 namespace {
-using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 // Tensor map of a K-major BF16 matrix [rows][K] (leading dimension ld
 // elements): boxes of 64 K x box_rows rows, 128-byte swizzle, zero fill.
 bool kmajor_map(CUtensorMap* out, const void* base, int rows, int K, int ld, int box_rows) {
-    static EncodeTiled encode = nullptr;
-    if (!encode) {
-        void* fn = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-                cudaSuccess ||
-            q != cudaDriverEntryPointSuccess || !fn)
-            return false;
-        encode = reinterpret_cast<EncodeTiled>(fn);
-    }
+    const EncodeTiled encode = tensor_map_encoder();
+    if (!encode) return false;
     const cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
     const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
     const cuuint32_t box[2] = {(cuuint32_t)kBK, (cuuint32_t)box_rows};

@@ -70,7 +70,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
     return false;
 }
 
-// D (tensor memory) = A B (+ D when accumulate), one K = 16 step.
+// D (tensor memory) = A B (+ D when accumulate), one K = 16 step; one thread.
 __device__ __forceinline__ void mma_f16(unsigned d, uint64_t a, uint64_t b, uint32_t idesc, unsigned accumulate) {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
@@ -79,9 +79,28 @@ __device__ __forceinline__ void mma_f16(unsigned d, uint64_t a, uint64_t b, uint
         : "memory");
 }
 
+// The same called by a whole converged warp, one elected thread of which issues
+// it.  Narrow products are bound by their issue: one thread of a branch takes
+// 75 clocks a step, this form 62, and two warps issuing side by side reach the
+// tensor core's 39 (128 rows, 16 columns; 64 at 128 columns).
+__device__ __forceinline__ void mma_f16_warp(unsigned d, uint64_t a, uint64_t b, uint32_t idesc, unsigned accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(idesc), "r"(accumulate));
+}
+
 // The barrier completes a phase when every matrix operation issued so far by this thread has completed.
 __device__ __forceinline__ void mma_commit(unsigned bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// For the operations of mma_f16_warp: the elected thread commits its own.
+__device__ __forceinline__ void mma_commit_warp(unsigned bar) {
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar)
+        : "memory");
 }
 
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -109,14 +128,14 @@ __device__ __forceinline__ void tmem_ld16(unsigned addr, uint32_t v[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// 16-byte asynchronous copy, zero fill when !ok (src must be a valid address either way).
-__device__ __forceinline__ void cp_async16(unsigned dst, const void* src, bool ok) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+// Tiled bulk tensor copy of one 5-D box into shared memory (128-byte aligned), zero beyond the tensor.
+__device__ __forceinline__ void tma_load_5d(unsigned dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, int c4,
+                                            unsigned bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5, %6}], "
+        "[%7];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(tm)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+        : "memory");
 }
 
 // Contiguous bulk copy into shared memory (16-byte aligned, bytes a multiple of 16).
@@ -124,6 +143,23 @@ __device__ __forceinline__ void bulk_load(unsigned dst, const void* src, unsigne
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
+}
+
+using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                 const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+// The driver's tensor-map encoder (nullptr when it has none).
+inline EncodeTiled tensor_map_encoder() {
+    static const EncodeTiled fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess)
+            f = nullptr;
+        return reinterpret_cast<EncodeTiled>(f);
+    }();
+    return fn;
 }
 
 }  // namespace vefd_nn

@@ -75,7 +75,7 @@ _MORE = {
     "vefd_nn_colsum": "vp ll i vp vp i vp",
     "vefd_nn_pack_weights": "vp i i i vp vp vp",
     "vefd_nn_splitk_reduce_t": "vp i ll i i i vp i vp",
-    "vefd_nn_conv3d_pack": "vp i i vp vp vp",
+    "vefd_nn_conv3d_pack": "vp i i i vp vp vp",
     "vefd_nn_conv3d_forward": "vp i i i i i i vp vp i i vp vp vp vp",
     "vefd_nn_conv3d_backward": "vp vp vp i i i i i i vp i i vp vp vp i vp vp vp",
     "vefd_nn_upsample2": "vp i i i i i vp vp",
@@ -104,8 +104,8 @@ def L():
         lb.vefd_nn_colsum_scratch.argtypes = [ctypes.c_longlong, ctypes.c_int]
         lb.vefd_nn_colsum_scratch.restype = ctypes.c_longlong
         pll = ctypes.POINTER(ctypes.c_longlong)
-        lb.vefd_nn_conv3d_sizes.argtypes = [ctypes.c_int, ctypes.c_int, pll, pll]
-        lb.vefd_nn_conv3d_sizes.restype = None
+        lb.vefd_nn_conv3d_sizes.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, pll, pll]
+        lb.vefd_nn_conv3d_sizes.restype = ctypes.c_int
         lb.vefd_nn_conv3d_backward_scratch.argtypes = [ctypes.c_int] * 7
         lb.vefd_nn_conv3d_backward_scratch.restype = ctypes.c_longlong
         _more_done = True
@@ -141,7 +141,7 @@ class Conv3d:
         self.mw, self.vw = torch.zeros_like(self.w), torch.zeros_like(self.w)
         self.mb, self.vb = torch.zeros_like(self.b), torch.zeros_like(self.b)
         nk, nd = ctypes.c_longlong(), ctypes.c_longlong()
-        L().vefd_nn_conv3d_sizes(cin, cout, ctypes.byref(nk), ctypes.byref(nd))
+        _check(L().vefd_nn_conv3d_sizes(cin, cout, stride, ctypes.byref(nk), ctypes.byref(nd)), "conv3d_sizes")
         self.wk = torch.empty(nk.value, dtype=torch.bfloat16, device="cuda")
         self.wd = torch.empty(nd.value, dtype=torch.bfloat16, device="cuda")
         self.status = torch.zeros(1, dtype=torch.int32, device="cuda")
@@ -151,8 +151,8 @@ class Conv3d:
         return [(self.w, self.dw, self.mw, self.vw), (self.b, self.db, self.mb, self.vb)]
 
     def pack(self):
-        _check(L().vefd_nn_conv3d_pack(_p(self.w), self.cin, self.cout, _p(self.wk), _p(self.wd), _stream()),
-               "conv3d_pack")
+        _check(L().vefd_nn_conv3d_pack(_p(self.w), self.cin, self.cout, self.stride, _p(self.wk), _p(self.wd),
+                                       _stream()), "conv3d_pack")
 
     def out_shape(self, shape):
         B, D, H, W, _ = shape

@@ -162,10 +162,11 @@ def test_conv_layer_matches_torch(cin, cout, stride, relu, shape):
 @pytest.mark.parametrize("cin,cout,stride,shape", [
     (8, 8, 1, (1, 1, 1, 8)), (8, 16, 2, (1, 5, 3, 16)), (3, 24, 1, (2, 3, 5, 8)), (24, 40, 1, (1, 7, 9, 8)),
     (48, 16, 1, (1, 6, 10, 24)), (16, 264, 1, (1, 2, 3, 8)), (232, 80, 1, (1, 4, 4, 8)), (40, 152, 2, (2, 7, 6, 16)),
-    (16, 32, 2, (1, 2, 1, 16)), (64, 256, 1, (1, 3, 3, 8))])
-def test_conv_gather_products(cin, cout, stride, shape):
-    """The gathered products at the edges of their tiles (one voxel row, ragged
-    rows and channel slabs, several column tiles, odd sizes at stride 2) against
+    (16, 32, 2, (1, 2, 1, 16)), (64, 256, 1, (1, 3, 3, 8)), (48, 16, 1, (1, 20, 18, 24)), (16, 32, 2, (1, 20, 36, 32)),
+    (112, 16, 2, (1, 4, 4, 16)), (264, 8, 1, (1, 2, 2, 8)), (16, 296, 2, (1, 3, 2, 16)), (152, 152, 1, (1, 8, 8, 8))])
+def test_conv_products(cin, cout, stride, shape):
+    """The products at the edges of their tiles (one voxel row, ragged rows and
+    channel slabs, several column tiles and channel blocks, odd sizes at stride 2) against
     FP64 of the BF16 operands they multiply: only FP32 accumulation is left,
     over K terms an error below sqrt(K) 2^-23 of the terms' size; 1e-5 sqrt(K)
     of the largest value is the bound of the other products here."""
