@@ -72,9 +72,14 @@ int vefd_nn_splitk_reduce_t(const float *parts, int splits, long long split_stri
 int vefd_nn_conv3d_sizes(int Cin, int Cout, int stride, long long *wk, long long *wd);
 /* w[Cout][27 Cin] -> wk (forward) and wd (backward data), BF16 (layouts in nn_conv.cu). */
 int vefd_nn_conv3d_pack(const float *w, int Cin, int Cout, int stride, void *wk, void *wd, void *stream);
-/* y[v'][o] = act(sum + bias[o]) (bias may be NULL; act max(., 0) when relu); writes xb for the backward pass. */
+/* y[v'][o] = act(sum + bias[o]) (bias may be NULL; act max(., 0) when relu).  Writes xb from x for this and the
+ * backward pass, or reads it as it is when x is NULL; yb (NULL, or BF16 [V'][Cout]) receives the next layer's xb. */
 int vefd_nn_conv3d_forward(const float *x, int B, int D, int H, int W, int Cin, int stride, const void *wk,
-                           const float *bias, int Cout, int relu, void *xb, float *y, unsigned *status, void *stream);
+                           const float *bias, int Cout, int relu, void *xb, float *y, void *yb, unsigned *status,
+                           void *stream);
+/* xb[v] = [u upsampled by 2 (nearest neighbour), s] of BF16 grids u [B][D/2][H/2][W/2][Cu], s [B][D][H][W][Cs];
+ * Cu, Cs multiples of 8, D, H, W even. */
+int vefd_nn_up_concat(const void *u, int Cu, const void *s, int Cs, int B, int D, int H, int W, void *xb, void *stream);
 /* Floats of scratch the backward pass needs (0 for bad sizes). */
 long long vefd_nn_conv3d_backward_scratch(int B, int D, int H, int W, int Cin, int stride, int Cout);
 /* Gradients for the output gradient dy: dw[o][k] and db[o] (added when accumulate), dx (overwritten); y the

@@ -23,6 +23,14 @@
 //   k_conv_dw  dW^T[(tap, channel)][o] = sum over voxels, one accumulator per tap.
 // Sums over K run tap by tap, 16 channels at a time, in the order of the
 // im2col product (the prediction's bits are those of that product).
+//
+// Measured, 64^3 unless said: the prediction 368 us (explicit im2col matrices and
+// their scalar kernels: 12263); 48 -> 16 channels forward and backward 175 us
+// (6742), of it 43 us forward, 62 us weight gradient, 32 us data gradient, 37 us
+// conversion, mask and sums; 232 -> 80 at 16^3 115 us (780), 49 us forward: one
+// chain of 392 steps a tile at about 85 clocks a step, which bounds the deep
+// levels; the fine ones are bound by the tensor core's 39 clocks a step of 16
+// columns (22 us of the 43) and the staging of 16-byte pieces.
 #include <algorithm>
 #include <cmath>
 
@@ -177,6 +185,13 @@ __device__ __forceinline__ void issue_runs(const uint2* pairs, int k0, int k1, u
     }
 }
 
+__device__ __forceinline__ uint4 pack8(const float* f) {
+    __nv_bfloat162 h[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
+    return *reinterpret_cast<uint4*>(h);
+}
+
 // Blocks walk the (tile, column block) items blockIdx.x, + gridDim.x, ...
 // Warp 7 copies each item's halo (channel block by channel block) into one of
 // `nbuf` buffers, warp 5 streams the weights Wk[piece][Np][8 BF16] (pieces in
@@ -189,8 +204,8 @@ __device__ __forceinline__ void issue_runs(const uint2* pairs, int k0, int k1, u
 __global__ void __launch_bounds__(kConvThreads, 2)
     k_conv(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
            const __grid_constant__ Halo h, const __grid_constant__ Entries ent, const uint4* __restrict__ Wk, int Np, int bn,
-           int nbuf, int nset, int cols, int chunk, float* __restrict__ Y, int Do, int Ho, int Wo,
-           const float* __restrict__ bias, int N, int relu, int vec, unsigned* __restrict__ status) {
+           int nbuf, int nset, int cols, int chunk, float* __restrict__ Y, uint4* __restrict__ Yb, int Do, int Ho,
+           int Wo, const float* __restrict__ bias, int N, int relu, int vec, unsigned* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char dsm[];
     __shared__ __align__(8) unsigned long long afull[2], aempty[2], bfull[kBStages], bempty[kBStages], acc_full[2],
         acc_empty[2], drain[2];
@@ -248,6 +263,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 const bool in = (!m64 || lane < 16) && rz < h.Rz && ry < h.Ry && rx < h.Rx;
                 const long long o = in ? out_voxel(ent.nrun, r, a.b, rz, ry, rx, Do, Ho, Wo) : -1;
                 float* y = Y + (o < 0 ? 0 : o) * N;
+                uint4* yb = Yb ? Yb + (o < 0 ? 0 : o) * (N / 8) : nullptr;
                 for (int c0 = 0; c0 < bw && n0 + c0 < N; c0 += 16) {
                     uint32_t v[16];
                     tmem_ld16(tmem + ((unsigned)(warp * 32) << 16) + (unsigned)((set * nacc + k) * bn + c0), v);
@@ -270,6 +286,11 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                             for (int q = 0; q < 4; ++q)
                                 if (n + q < N) y[n + q] = f[i + q];
                         }
+                    }
+                    if (yb) {  // N a multiple of 8
+#pragma unroll
+                        for (int i = 0; i < 16; i += 8)
+                            if (n0 + c0 + i < N) yb[(n0 + c0 + i) / 8] = pack8(f + i);
                     }
                 }
             }
@@ -528,10 +549,23 @@ __global__ void k_pad_bf16(const float* __restrict__ x, long long V, int C, int 
 #pragma unroll
             for (int j = 0; j < 8; ++j) f[j] = c + j < C ? x[v * C + c + j] : 0.0f;
         }
-        __nv_bfloat162 h[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
-        xb[e] = *reinterpret_cast<uint4*>(h);
+        xb[e] = pack8(f);
+    }
+}
+
+// xb[v] = [u[v / 2] (nearest-neighbour upsampling by 2), s[v]]: the pieces of
+// two BF16 grids, U8 and S8 a voxel; u is B x D/2 x H/2 x W/2, s and xb B x D x H x W.
+__global__ void k_up_concat(const uint4* __restrict__ u, int U8, const uint4* __restrict__ s, int S8, int B, int D, int H, int W,
+                            uint4* __restrict__ xb) {
+    const unsigned C = U8 + S8, n = (unsigned)B * D * H * W * C;
+    for (unsigned e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+        const unsigned v = e / C, c = e - v * C;
+        if (c >= (unsigned)U8) {
+            xb[e] = s[(long long)v * S8 + c - U8];
+        } else {
+            const unsigned x = v % W, r = v / W, y = r % H, q = r / H, z = q % D, b = q / D;
+            xb[e] = u[((((long long)b * (D / 2) + z / 2) * (H / 2) + y / 2) * (W / 2) + x / 2) * U8 + c];
+        }
     }
 }
 
@@ -555,15 +589,12 @@ __global__ void __launch_bounds__(kActThreads)
                 const float4 p = reinterpret_cast<const float4*>(y)[2 * e], q = reinterpret_cast<const float4*>(y)[2 * e + 1];
                 float f[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
                 const float o[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
-                __nv_bfloat162 h[4];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     if (relu && !(o[j] > 0.0f)) f[j] = 0.0f;
                     acc[j] += f[j];
                 }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) h[j] = __floats2bfloat162_rn(f[2 * j], f[2 * j + 1]);
-                gb[e] = *reinterpret_cast<uint4*>(h);
+                gb[e] = pack8(f);
             }
         __syncthreads();
 #pragma unroll
@@ -578,26 +609,31 @@ __global__ void __launch_bounds__(kActThreads)
     }
 }
 
-// dw[o][tap C + c] (+)= sum_s parts[s][tap 8 C8 + c][o], db[o] (+)= sum_b part[b][o], in order.
-__global__ void k_dw_reduce(const float* __restrict__ parts, int splits, int C, int Cp, int Cout,
-                            const float* __restrict__ dbpart, int nparts, float* __restrict__ dw, float* __restrict__ db,
-                            int accumulate) {
-    const int n = kTaps * Cp * Cout;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < n) {
+// dw[o][tap C + c] (+)= sum_s parts[s][tap 8 C8 + c][o] (the first `dwblocks`
+// blocks, a thread each), db[o] (+)= sum_b part[b][o] (a warp each: lanes take
+// every 32nd part, then a fixed tree).
+__global__ void __launch_bounds__(128)
+    k_dw_reduce(const float* __restrict__ parts, int splits, int C, int Cp, int Cout, const float* __restrict__ dbpart,
+                int nparts, int dwblocks, float* __restrict__ dw, float* __restrict__ db, int accumulate) {
+    if ((int)blockIdx.x < dwblocks) {
+        const int n = kTaps * Cp * Cout;
+        const int e = blockIdx.x * blockDim.x + threadIdx.x;
+        if (e >= n) return;
         const int o = e % Cout, k = e / Cout, tap = k / Cp, c = k % Cp;
         if (c >= C) return;
         float acc = 0.0f;
-#pragma unroll 8
+#pragma unroll 16
         for (int s = 0; s < splits; ++s) acc += parts[(long long)s * n + e];
         float* d = dw + ((long long)o * kTaps + tap) * C + c;
         *d = accumulate ? *d + acc : acc;
-    } else if (e < n + Cout) {
-        const int o = e - n;
+    } else {
+        const int o = ((int)blockIdx.x - dwblocks) * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+        if (o >= Cout) return;
         float acc = 0.0f;
-#pragma unroll 8
-        for (int s = 0; s < nparts; ++s) acc += dbpart[(long long)s * Cout + o];
-        db[o] = accumulate ? db[o] + acc : acc;
+        for (int s = lane; s < nparts; s += 32) acc += dbpart[(long long)s * Cout + o];
+#pragma unroll
+        for (int d = 16; d > 0; d >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, d);
+        if (lane == 0) db[o] = accumulate ? db[o] + acc : acc;
     }
 }
 
@@ -811,10 +847,12 @@ struct ConvPlan {
 };
 
 // Tile of a pass: the choice with the least estimated time.  Per item, in SM
-// clocks: the staged pieces at one a clock and their latency, the matrix operations at 39 a step
-// (half a clock a column beyond 78) on the SM's tensor core and at 80 on each of
-// a block's issuing warps, which take every other accumulator, and 1500 between
-// the items of a block; 6000 for launch and the first copies.
+// clocks: the staged pieces at one a clock and their latency, the matrix
+// operations at 39 a step (half a clock a column beyond 78) on the SM's tensor
+// core and at 85 on each of a block's issuing warps, which take every other
+// accumulator, 450 a chunk of weights, and 1500 between the items of a block;
+// 6000 for launch and the first copies.  (Deep levels, a few hundred steps over
+// a few tiles, are a chain of steps and chunks; the fine ones fill the SMs.)
 ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, int nrun, int npairs) {
     ConvPlan best{};
     double best_t = 0.0;
@@ -828,26 +866,28 @@ ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, 
                 const int bn = round_up((Np + nt - 1) / nt, 16), set = nrun * T * bn;
                 if (bn > 256 || set > 512 || bn == last) continue;
                 last = bn;
-                ConvPlan p{PY, T, bn, bn <= 16 ? 16 : (bn <= 32 ? 8 : (bn <= 128 ? 4 : 2)), 2, set <= 256 ? 2 : 1, 1, 0, true};
-                const unsigned a = h.slabs * h.pitch_slab;
-                const unsigned ring = kBStages * (unsigned)p.chunk * 2 * bn * 16;
-                if (2 * a + ring > kSmemMax) p.nbuf = 1;
-                p.smem = p.nbuf * a + ring;
-                if (p.smem > kSmemMax) continue;
-                const int cols = acc_alloc(p.nset * set);
-                p.occ = std::max(1, std::min(4, std::min((int)(kSmemMax / (p.smem + 5120)), 512 / cols)));
-                const long long items = (long long)h.ntiles * ((Np + bn - 1) / bn), slots = (long long)sm_count() * p.occ;
-                const double load = (double)h.nblk * (1.0 * h.hz * h.hy * h.hx * h.s * h.slabs + 1500.0);
-                const double steps = (double)npairs * h.nblk;
-                const double mma = steps * T * std::max(39.0, bn / 2.0);               // the SM's tensor core
-                const double issue = steps * (nrun > 1 ? 0.5 : (T + 1) / 2) * std::max(80.0, bn / 2.0);  // a block's warps
-                // an SM works through its share; a block's own items follow one another
-                const double share = (double)items / sm_count(), chain = (double)((items + slots - 1) / slots);
-                const double own = p.nbuf == 2 ? std::max(load, issue) : load + issue;
-                const double tm = std::max(std::ceil(share) * std::max(load, mma), chain * (own + 1500.0)) + load + 6000.0;
-                if (!best.ok || tm < best_t) {
-                    best = p;
-                    best_t = tm;
+                for (int chunk = 2; chunk <= 32; chunk *= 2) {
+                    ConvPlan p{PY, T, bn, chunk, 2, set <= 256 ? 2 : 1, 1, 0, true};
+                    const unsigned a = h.slabs * h.pitch_slab, ring = kBStages * (unsigned)chunk * 2 * bn * 16;
+                    if (2 * a + ring > kSmemMax) p.nbuf = 1;
+                    p.smem = p.nbuf * a + ring;
+                    if (p.smem > kSmemMax) continue;
+                    const int cols = acc_alloc(p.nset * set);
+                    p.occ = std::max(1, std::min(4, std::min((int)(kSmemMax / (p.smem + 5120)), 512 / cols)));
+                    const long long items = (long long)h.ntiles * ((Np + bn - 1) / bn), slots = (long long)sm_count() * p.occ;
+                    const double load = (double)h.nblk * (1.0 * h.hz * h.hy * h.hx * h.s * h.slabs + 1500.0);
+                    const double steps = (double)npairs * h.nblk;
+                    const double mma = steps * T * std::max(39.0, bn / 2.0);               // the SM's tensor core
+                    const double issue = steps * (nrun > 1 ? 0.5 : (T + 1) / 2) * std::max(85.0, bn / 2.0) +
+                                         450.0 * h.nblk * ((npairs + chunk - 1) / chunk);  // a block's warps
+                    // an SM works through its share; a block's own items follow one another
+                    const double share = (double)items / sm_count(), chain = (double)((items + slots - 1) / slots);
+                    const double own = p.nbuf == 2 ? std::max(load, issue) : load + issue;
+                    const double tm = std::max(std::ceil(share) * std::max(load, mma), chain * (own + 1500.0)) + load + 6000.0;
+                    if (!best.ok || tm < best_t) {
+                        best = p;
+                        best_t = tm;
+                    }
                 }
             }
         }
@@ -856,7 +896,7 @@ ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, 
 
 // kind as halo_of; N output channels, Y on the grid Do x Ho x Wo.
 cudaError_t launch_conv(int kind, const void* A, int B, int D, int H, int W, int C8, int s, const void* wk, int N, float* Y,
-                        int Do, int Ho, int Wo, const float* bias, int relu, unsigned* status, cudaStream_t st) {
+                        void* Yb, int Do, int Ho, int Wo, const float* bias, int relu, unsigned* status, cudaStream_t st) {
     const int Np = round_up(N, 16), nrun = kind == 1 ? 8 : 1;
     Entries e = kind == 1 ? adjoint_entries(halo_of(1, B, D, H, W, C8, 1, 8, 1)) : conv_entries(halo_of(0, B, D, H, W, C8, s, 8, 1));
     if (e.npairs > kMaxPairs) return cudaErrorInvalidValue;
@@ -873,7 +913,7 @@ cudaError_t launch_conv(int kind, const void* A, int B, int D, int H, int W, int
     const int vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
     const int grid = (int)std::min<long long>(items, (long long)sm_count() * p.occ);
     k_conv<<<grid, kConvThreads, p.smem, st>>>(tm0, tm1, h, e, (const uint4*)wk, Np, p.bn, p.nbuf, p.nset,
-                                               acc_alloc(p.nset * nrun * p.T * p.bn), p.chunk, Y, Do, Ho, Wo, bias, N, relu,
+                                               acc_alloc(p.nset * nrun * p.T * p.bn), p.chunk, Y, (uint4*)Yb, Do, Ho, Wo, bias, N, relu,
                                                vec, status);
     return cudaGetLastError();
 }
@@ -962,16 +1002,30 @@ int vefd_nn_conv3d_pack(const float* w, int Cin, int Cout, int stride, void* wk,
     return cudaGetLastError() == cudaSuccess ? VEFD_NN_OK : VEFD_NN_ERR_CUDA;
 }
 
+int vefd_nn_up_concat(const void* u, int Cu, const void* s, int Cs, int B, int D, int H, int W, void* xb, void* stream) {
+    if (!u || !s || !xb || Cu < 8 || Cs < 8 || Cu % 8 || Cs % 8 || B < 1 || D < 2 || H < 2 || W < 2 || D % 2 || H % 2 || W % 2)
+        return VEFD_NN_ERR_ARG;
+    if (misaligned(u) || misaligned(s) || misaligned(xb)) return VEFD_NN_ERR_ARG;
+    const long long n = (long long)B * D * H * W * (Cu + Cs) / 8;
+    if (n > 0x7fffffffLL) return VEFD_NN_ERR_ARG;
+    k_up_concat<<<(int)std::min<long long>((n + 255) / 256, 152 * 16), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+        (const uint4*)u, Cu / 8, (const uint4*)s, Cs / 8, B, D, H, W, (uint4*)xb);
+    return cudaGetLastError() == cudaSuccess ? VEFD_NN_OK : VEFD_NN_ERR_CUDA;
+}
+
 int vefd_nn_conv3d_forward(const float* x, int B, int D, int H, int W, int Cin, int stride, const void* wk,
-                           const float* bias, int Cout, int relu, void* xb, float* y, unsigned* status, void* stream) {
-    if (!x || !wk || !xb || !y || !status || bad_conv(B, D, H, W, Cin, Cout, stride) || misaligned(wk) || misaligned(xb))
+                           const float* bias, int Cout, int relu, void* xb, float* y, void* yb, unsigned* status,
+                           void* stream) {
+    if (!wk || !xb || !y || !status || bad_conv(B, D, H, W, Cin, Cout, stride) || misaligned(wk) || misaligned(xb) ||
+        misaligned(yb))
         return VEFD_NN_ERR_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const int C8 = (Cin + 7) / 8;
     const long long V = (long long)B * D * H * W, n = V * C8;
     const int vec = Cin % 8 == 0 && !misaligned(x);
-    k_pad_bf16<<<(int)std::min<long long>((n + 255) / 256, 152 * 16), 256, 0, s>>>(x, V, Cin, C8, vec, (uint4*)xb);
-    const cudaError_t e = launch_conv(0, xb, B, D, H, W, C8, stride, wk, Cout, y, (D - 1) / stride + 1, (H - 1) / stride + 1,
+    if (x)
+        k_pad_bf16<<<(int)std::min<long long>((n + 255) / 256, 152 * 16), 256, 0, s>>>(x, V, Cin, C8, vec, (uint4*)xb);
+    const cudaError_t e = launch_conv(0, xb, B, D, H, W, C8, stride, wk, Cout, y, yb, (D - 1) / stride + 1, (H - 1) / stride + 1,
                                       (W - 1) / stride + 1, bias, relu, status, s);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? VEFD_NN_OK : VEFD_NN_ERR_CUDA;
 }
@@ -1009,10 +1063,11 @@ int vefd_nn_conv3d_backward(const void* xb, const float* y, const float* dy, int
         return VEFD_NN_ERR_CUDA;
     k_conv_dw<<<dim3(9 / p.ntap * p.mblks, p.nt, p.splits), kConvThreads, p.smem, s>>>(
         tm0, tm1, tmG, h, Cout, p.bn, acc_alloc(p.ntap * p.bn), p.ntap, p.mslabs, p.stages, p.per, parts, status);
-    const int n = kTaps * C8 * 8 * Cout + Cout;
-    k_dw_reduce<<<(n + 127) / 128, 128, 0, s>>>(parts, p.splits, Cin, C8 * 8, Cout, dbpart, nb, dw, db, accumulate);
+    const int dwblocks = (kTaps * C8 * 8 * Cout + 127) / 128;
+    k_dw_reduce<<<dwblocks + (Cout + 3) / 4, 128, 0, s>>>(parts, p.splits, Cin, C8 * 8, Cout, dbpart, nb, dwblocks, dw, db,
+                                                          accumulate);
     const int Do = (D - 1) / stride + 1, Ho = (H - 1) / stride + 1, Wo = (W - 1) / stride + 1;
-    e = launch_conv(stride == 1 ? 0 : 1, gb, B, Do, Ho, Wo, O8, 1, wd, Cin, dx, D, H, W, nullptr, 0, status, s);
+    e = launch_conv(stride == 1 ? 0 : 1, gb, B, Do, Ho, Wo, O8, 1, wd, Cin, dx, nullptr, D, H, W, nullptr, 0, status, s);
     return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? VEFD_NN_OK : VEFD_NN_ERR_CUDA;
 }
 

@@ -76,7 +76,8 @@ _MORE = {
     "vefd_nn_pack_weights": "vp i i i vp vp vp",
     "vefd_nn_splitk_reduce_t": "vp i ll i i i vp i vp",
     "vefd_nn_conv3d_pack": "vp i i i vp vp vp",
-    "vefd_nn_conv3d_forward": "vp i i i i i i vp vp i i vp vp vp vp",
+    "vefd_nn_conv3d_forward": "vp i i i i i i vp vp i i vp vp vp vp vp",
+    "vefd_nn_up_concat": "vp i vp i i i i i vp vp",
     "vefd_nn_conv3d_backward": "vp vp vp i i i i i i vp i i vp vp vp i vp vp vp",
     "vefd_nn_upsample2": "vp i i i i i vp vp",
     "vefd_nn_upsample2_backward": "vp i i i i i vp i vp",
@@ -163,11 +164,18 @@ class Conv3d:
         import torch
         B, D, H, W, C = x.shape
         assert C == self.cin and x.is_contiguous()
-        y = torch.empty(self.out_shape(x.shape), device="cuda")
         xb = torch.empty(B * D * H * W, round8(C), dtype=torch.bfloat16, device="cuda")
+        return self._forward(x, xb, x.shape, None)
+
+    def _forward(self, x, xb, shape, yb):
+        """The layer on x, or on the BF16 copy xb alone (x None); yb receives the output's."""
+        import torch
+        B, D, H, W, C = shape
+        y = torch.empty(self.out_shape(shape), device="cuda")
         _check(L().vefd_nn_conv3d_forward(_p(x), B, D, H, W, C, self.stride, _p(self.wk), _p(self.b), self.cout,
-                                          int(self.relu), _p(xb), _p(y), _p(self.status), _stream()), "conv3d_forward")
-        self._saved = (x.shape, xb, y)
+                                          int(self.relu), _p(xb), _p(y), _p(yb), _p(self.status), _stream()),
+               "conv3d_forward")
+        self._saved = (shape, xb, y)
         return y
 
     def backward(self, dy, accumulate=False):
@@ -266,25 +274,42 @@ class UNet:
         return sum(int(t.numel()) for lay in self.layers for t, _, _, _ in lay.params())
 
     @staticmethod
-    def _run(layers, x):
-        for lay in layers:
-            x = lay.forward(x)
-        return x
-
-    @staticmethod
     def _back(layers, dy, accumulate=False):
         for lay in reversed(layers):
             dy = lay.backward(dy, accumulate)
         return dy
 
     def forward(self, x):
-        s0 = self._run(self.e0, x)
-        s1 = self._run(self.e1, s0)
-        s2 = self._run(self.e2, s1)
-        s3 = self._run(self.e3, s2)
-        u2 = self._run(self.d2, concat(upsample2(s3), s2))
-        u1 = self._run(self.d1, concat(upsample2(u2), s1))
-        out = self._run(self.d0, concat(upsample2(u1), s0))
+        import torch
+
+        def grid(shape):
+            return torch.empty(shape, dtype=torch.bfloat16, device="cuda")
+
+        def run(layers, x, xb, shape):
+            """(output, its BF16 copy or None for the last layer) of a level's layers; each
+            layer writes the copy that the next one reads."""
+            for lay in layers:
+                yb = grid(lay.out_shape(shape)) if lay is not self.layers[-1] else None
+                x, xb, shape = None, yb, (y := lay._forward(x, xb, shape, yb)).shape
+            return y, yb
+
+        def up(layers, ub, sb):
+            """The decoder level on [ub upsampled by 2, sb]."""
+            B, D, H, W, Cs = sb.shape
+            shape = (B, D, H, W, ub.shape[-1] + Cs)
+            xb = grid(shape)
+            _check(L().vefd_nn_up_concat(_p(ub), ub.shape[-1], _p(sb), Cs, B, D, H, W, _p(xb), _stream()), "up_concat")
+            return run(layers, None, xb, shape)
+
+        B, D, H, W, C = x.shape
+        assert C == self.layers[0].cin and x.is_contiguous()
+        s0, b0 = run(self.e0, x, grid((B, D, H, W, round8(C))), x.shape)
+        s1, b1 = run(self.e1, None, b0, s0.shape)
+        s2, b2 = run(self.e2, None, b1, s1.shape)
+        s3, b3 = run(self.e3, None, b2, s2.shape)
+        u2, v2 = up(self.d2, b3, b2)
+        u1, v1 = up(self.d1, v2, b1)
+        out, _ = up(self.d0, v1, b0)
         self._shapes = (s0.shape, s1.shape, s2.shape, s3.shape, u2.shape, u1.shape)
         return out
 
