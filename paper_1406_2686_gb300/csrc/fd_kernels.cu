@@ -333,21 +333,29 @@ __device__ __forceinline__ void store_feedback(const float c[L::NC], const float
 // time n to n+1 when the polymer is evolved, and the feedback stress of time
 // n+1 for the next lattice step.  All of it only reads data the lattice kernel
 // has finished writing, so one pass over the lattice does it.
+// One thread per node over runs of 128 consecutive nodes (x fastest), so no lane
+// is spent on the padding of a box; stencil neighbours come from L1 and L2.
+// Bound by the latency of its 107 loads a node: five blocks per SM (102
+// registers) measure 25.1 us on 100 x 50 x 70 FP32 against 28.8 without the
+// bound, 26.1 with 6 and 28.5 with 8.  32 x 4 x 2 boxes with the populations
+// staged by a tensor copy, which the run form replaced, took 33.1 us there, 20.6
+// against 18.1 on 88 x 48 x 64 and 19.4 against 16.8 on 64^3.
+constexpr int kPostBlocks = 5;
+
 template <class PT, class L, int NCOMP, bool FD>
-__global__ void __launch_bounds__(128) k_post(const PT* __restrict__ fnew, const float* __restrict__ frest,
+__global__ void __launch_bounds__(128, kPostBlocks) k_post(const PT* __restrict__ fnew, const float* __restrict__ frest,
                                               float* __restrict__ drho,
                                               const float* __restrict__ Ct, float* __restrict__ Cout,
                                               float* __restrict__ R, const float* __restrict__ u,
                                               float* __restrict__ Q, unsigned* __restrict__ status, StepParams p,
                                               int rev) {
-    const int bxi = rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-    const int byi = rev ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
-    const int x = bxi * blockDim.x + threadIdx.x;
-    const int y = byi * blockDim.y + threadIdx.y;
-    const int z = rev ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z;
-    if (x >= p.nx || y >= p.ny) return;
+    // everything below reads or overwrites data of the preceding lattice kernel
+    pdl_wait();
     const long long N = p.N;
-    const long long i = ((long long)z * p.ny + y) * p.nx + x;
+    const int i = (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * 128 + threadIdx.x;
+    if (i >= N) return;
+    const int row = (int)((unsigned)i / (unsigned)p.nx), x = i - row * p.nx;
+    const int z = (int)((unsigned)row / (unsigned)p.ny), y = row - z * p.ny;
     float d[NCOMP];
 #pragma unroll
     for (int s = 0; s < NCOMP; ++s) {
@@ -362,68 +370,7 @@ __global__ void __launch_bounds__(128) k_post(const PT* __restrict__ fnew, const
 #pragma unroll
         for (int k = 0; k < L::NC; ++k) c[k] = __ldg(Ct + k * N + i);
     }
-    dens_store<NCOMP>(drho, i, d);
-    if (p.feedback != 0.0f) store_feedback<L, NCOMP>(c, d, p, Q, N, i);
-}
-
-// The same pass with the tile's new populations staged in shared memory by
-// one bulk tensor copy, issued before the stencil loads so that both are in
-// flight together; the densities are summed from shared memory afterwards in
-// the same order.
-template <class PT, class L, int NCOMP, bool FD, int BX, int BY, int BZ>
-__global__ void __launch_bounds__(BX * BY * BZ) k_post_tma(const __grid_constant__ CUtensorMap tm_fnew,
-                                                           const float* __restrict__ frest,
-                                                           float* __restrict__ drho, const float* __restrict__ Ct,
-                                                           float* __restrict__ Cout, float* __restrict__ R,
-                                                           const float* __restrict__ u, float* __restrict__ Q,
-                                                           unsigned* __restrict__ status, StepParams p, int rev) {
-    constexpr int P = NCOMP * (L::Q - 1);  // moving populations
-    constexpr int T = BX * BY * BZ;
-    constexpr unsigned kBytes = (unsigned)(P * T * sizeof(PT));
-    extern __shared__ __align__(128) unsigned char sraw[];
-    PT* sf = reinterpret_cast<PT*>(sraw);  // [P][BZ][BY][BX]
-    __shared__ __align__(8) unsigned long long bar;
-    const int tx = threadIdx.x, ty = threadIdx.y, tz = threadIdx.z;
-    const int x0 = (rev ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x) * BX;
-    const int y0 = (rev ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y) * BY;
-    const int z0 = (rev ? (int)(gridDim.z - 1 - blockIdx.z) : (int)blockIdx.z) * BZ;
-    const bool leader = (tx | ty | tz) == 0;
-    const unsigned bar_a = smem_u32(&bar);
-    if (leader) mbar_init(bar_a);
-    __syncthreads();
-    if (leader) tma_load_4d(smem_u32(sf), &tm_fnew, x0, y0, z0, 0, bar_a, kBytes);
-    const int x = x0 + tx, y = y0 + ty, z = z0 + tz;
-    const bool active = x < p.nx && y < p.ny && z < p.nz;
-    const long long N = p.N;
-    const long long i = active ? ((long long)z * p.ny + y) * p.nx + x : 0;
-    float c[L::NC];
-    float rest[NCOMP];
-    if (active) {
-#pragma unroll
-        for (int s = 0; s < NCOMP; ++s) rest[s] = __ldg(frest + s * N + i);
-        if (FD) {
-            fenep_node<L::D, L::NC>(Ct, Cout, R, u, status, p, x, y, z, c);
-        } else {
-#pragma unroll
-            for (int k = 0; k < L::NC; ++k) c[k] = __ldg(Ct + k * N + i);
-        }
-    }
-    if (!mbar_wait_bounded(bar_a)) {
-        if (leader) {
-            atomicOr(status, kStTimeout);
-            mbar_wait_bounded(bar_a);  // bounded: let the copy land before leaving
-        }
-        return;
-    }
-    if (!active) return;
-    const int t = (tz * BY + ty) * BX + tx;
-    float d[NCOMP];
-#pragma unroll
-    for (int s = 0; s < NCOMP; ++s) {
-        d[s] = rest[s];
-#pragma unroll
-        for (int a = 1; a < L::Q; ++a) d[s] += pop_get(sf[(s * (L::Q - 1) + a - 1) * T + t]);
-    }
+    pdl_trigger();
     dens_store<NCOMP>(drho, i, d);
     if (p.feedback != 0.0f) store_feedback<L, NCOMP>(c, d, p, Q, N, i);
 }
@@ -729,16 +676,13 @@ __global__ void __launch_bounds__(128) k_pre(const PT* __restrict__ f, const flo
 
 cudaError_t launch_post(int lattice, int ncomp, bool fd, const StepParams& p, const StepBufs& b,
                         const void* fnew, cudaStream_t s, int rev) {
-    dim3 blk(32, 4, 1), grd((p.nx + 31) / 32, (p.ny + 3) / 4, p.nz);
+    const dim3 blk(128), grd((unsigned)((p.N + 127) / 128));
+    cudaError_t e = cudaSuccess;
 #define VEFD_POST(LT, NCP)                                                                                  \
     do {                                                                                                    \
         const PT* fn = static_cast<const PT*>(fnew);                                                        \
-        if (fd)                                                                                             \
-            k_post<PT, LT, NCP, true><<<grd, blk, 0, s>>>(fn, b.frest, b.drho, b.Cin, b.Cout, b.R, b.u, b.Q, b.status, p,  \
-                                                          rev);                                             \
-        else                                                                                                \
-            k_post<PT, LT, NCP, false><<<grd, blk, 0, s>>>(fn, b.frest, b.drho, b.Cin, b.Cout, b.R, b.u, b.Q, b.status, p, \
-                                                           rev);                                            \
+        e = launch_pdl(p.pdl != 0, fd ? k_post<PT, LT, NCP, true> : k_post<PT, LT, NCP, false>, grd, blk, 0, s, fn, \
+                       (const float*)b.frest, b.drho, b.Cin, b.Cout, b.R, (const float*)b.u, b.Q, b.status, p, rev); \
     } while (0)
     VEFD_WITH_PT(p.prec, {
         if (lattice == 1) {
@@ -750,36 +694,6 @@ cudaError_t launch_post(int lattice, int ncomp, bool fd, const StepParams& p, co
         }
     });
 #undef VEFD_POST
-    return cudaGetLastError();
-}
-
-namespace {
-template <class PT, class L, int NCOMP, int BX, int BY, int BZ>
-cudaError_t post_tma(bool fd, const CUtensorMap* tm, const StepParams& p, const StepBufs& b, cudaStream_t s, int rev) {
-    constexpr int smem = NCOMP * (L::Q - 1) * BX * BY * BZ * (int)sizeof(PT);
-    dim3 blk(BX, BY, BZ), grd((p.nx + BX - 1) / BX, (p.ny + BY - 1) / BY, (p.nz + BZ - 1) / BZ);
-    if (fd)
-        k_post_tma<PT, L, NCOMP, true, BX, BY, BZ><<<grd, blk, smem, s>>>(*tm, b.frest, b.drho, b.Cin, b.Cout, b.R, b.u, b.Q,
-                                                                           b.status, p, rev);
-    else
-        k_post_tma<PT, L, NCOMP, false, BX, BY, BZ><<<grd, blk, smem, s>>>(*tm, b.frest, b.drho, b.Cin, b.Cout, b.R, b.u, b.Q,
-                                                                            b.status, p, rev);
-    return cudaGetLastError();
-}
-}  // namespace
-
-cudaError_t launch_post_tma(int lattice, int ncomp, bool fd, const StepParams& p, const StepBufs& b,
-                            const void* tensor_map_fnew, cudaStream_t s, int rev) {
-    const CUtensorMap* tm = static_cast<const CUtensorMap*>(tensor_map_fnew);
-    cudaError_t e = cudaSuccess;
-    VEFD_WITH_PT(p.prec, {
-        if (lattice == 1)
-            e = ncomp == 2 ? post_tma<PT, D3Q19, 2, 32, 4, 2>(fd, tm, p, b, s, rev)
-                           : post_tma<PT, D3Q19, 1, 32, 4, 2>(fd, tm, p, b, s, rev);
-        else
-            e = ncomp == 2 ? post_tma<PT, D2Q9, 2, 32, 8, 1>(fd, tm, p, b, s, rev)
-                           : post_tma<PT, D2Q9, 1, 32, 8, 1>(fd, tm, p, b, s, rev);
-    });
     return e;
 }
 

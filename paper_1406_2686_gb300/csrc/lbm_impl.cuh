@@ -515,14 +515,122 @@ __device__ __forceinline__ void collide_stream(const StepBufs& b, const StepPara
     }
 }
 
-template <class PT, class L, int NCOMP, bool STREAM, int COLL>
-__global__ void __launch_bounds__(128) k_lattice(StepBufs b, StepParams p, int rev) {
-    const int x = tile_index(blockIdx.x, gridDim.x, rev) * blockDim.x + threadIdx.x;
-    const int y = tile_index(blockIdx.y, gridDim.y, rev) * blockDim.y + threadIdx.y;
-    const int z = tile_index(blockIdx.z, gridDim.z, rev);
-    if (x >= p.nx || y >= p.ny) return;
+// --- TMA-staged variant --------------------------------------------------------
+
+// Threads per SM the register budget of the staged lattice kernel is sized
+// for (1024: 64 registers per thread).
+#ifndef VEFD_LATTICE_THREADS_PER_SM
+#define VEFD_LATTICE_THREADS_PER_SM 1024
+#endif
+
+// Node work of the staged kernels, split around the wait for the staged
+// populations: gather (neighbour densities and feedback stress, overlapping
+// the copy), then moments, local state and collision from shared memory.
+template <class L, int NCOMP>
+struct NodeGather {
+    float dr[NCOMP];
+    float acc[2][3], Fp[3], qloc[L::NQ];
+    Nbr nb;
+};
+
+template <class L, int NCOMP>
+__device__ __forceinline__ void node_gather(const StepBufs& b, const StepParams& p, int x, int y, int z, bool active,
+                                            NodeGather<L, NCOMP>& g) {
+    g.nb = make_nbr(active ? x : 0, active ? y : 0, active ? z : 0, p);
+    if (!active) return;
+    // the node's own deviations come from the density buffer (bit-identical to
+    // the sum of the staged populations)
+    dens_ldg<NCOMP>(b.drho, g.nb.i, g.dr);
+    neighbour_forces<L, NCOMP>(b, p, g.nb, g.acc, g.Fp, g.qloc);
+}
+
+// Moments, local state and collision of one node: `first` reads a moving
+// population for the moments, `again` reads it for the collision.  TRIGGER lets
+// the next kernel of the stream launch before the stores.
+template <class PT, class L, int NCOMP, int COLL, bool EDGE = true, bool PARTS = false, bool TRIGGER = true,
+          class First, class Again>
+__device__ __forceinline__ void node_collide(const StepBufs& b, const StepParams& p, const NodeGather<L, NCOMP>& g,
+                                             First first, Again again, PT* own = nullptr, int T = 0,
+                                             float* rest_out = nullptr) {
     const long long N = p.N;
-    const long long i = ((long long)z * p.ny + y) * p.nx + x;
+    const int i = g.nb.i;
+    float jx = 0.0f, jy = 0.0f, jz = 0.0f;
+    float pif[NCOMP][6];
+#pragma unroll
+    for (int s = 0; s < NCOMP; ++s) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) pif[s][k] = 0.0f;
+#pragma unroll
+        for (int a = 1; a < L::Q; ++a) {
+            const float fa = first(s, a);
+            if (L::cx(a)) jx += L::cx(a) * fa;
+            if (L::cy(a)) jy += L::cy(a) * fa;
+            if (L::cz(a)) jz += L::cz(a) * fa;
+            if (COLL == 1) pi_add<L>(pif[s], a, fa);
+        }
+    }
+    Local<NCOMP> st;
+    local_state<L, NCOMP>(p, g.dr, jx, jy, jz, g.acc, g.Fp, st, b.status);
+    b.u[i] = st.ux;
+    b.u[N + i] = st.uy;
+    if (L::D == 3) b.u[2 * N + i] = st.uz;
+    if (TRIGGER) pdl_trigger();
+    collide_stream<PT, L, NCOMP, COLL, EDGE, PARTS>(b, p, g.nb, st, g.qloc, pif, again, own, T, rest_out);
+}
+
+// The same with the tile's populations in shared memory (sf[plane * T + t]).
+template <class PT, class L, int NCOMP, int T, int COLL, bool EDGE = true, bool PARTS = false>
+__device__ __forceinline__ void node_collide(const StepBufs& b, const StepParams& p, const PT* sf, int t,
+                                             const NodeGather<L, NCOMP>& g, PT* own = nullptr,
+                                             float* rest_out = nullptr) {
+    // volatile reads keep the populations in shared memory instead of registers
+    node_collide<PT, L, NCOMP, COLL, EDGE, PARTS, false>(
+        b, p, g, [&](int s, int a) { return pop_get(sf[(s * (L::Q - 1) + a - 1) * T + t]); },
+        [&](int s, int a) { return pop_smem(sf, (s * (L::Q - 1) + a - 1) * T + t); }, own, T, rest_out);
+}
+
+// Resident 128-thread blocks per SM the register kernel is compiled for.
+// Measured on D3Q19, two components: 5 (96 registers) against the 3 blocks
+// that 168 registers allow, and 4 and 6: 100 x 50 x 70 27.4 us (4: 29.7, 6:
+// 29.3).  The FP32 moment-space collision, which reads its populations twice
+// (see k_lattice), takes 6: the same box 25.1 us (5: 26.3, 7: 26.3).  16-bit
+// storage takes 4 (24.7 us, 5: 24.2, 3: 26.7): at 96 registers the compiler
+// rounds the moving-wall term in another order than in the staged kernels, which
+// 16-bit storage turns into flipped last bits.
+template <class PT, class L, int COLL>
+constexpr int reg_blocks() {
+    return sizeof(PT) == 2 ? 4 : L::D == 3 && COLL == 1 ? 6 : 5;
+}
+
+// The step with one thread per node over runs of 128 consecutive nodes (x
+// fastest), whatever the lattice's shape: every lane of every block but the
+// last one has a node, while 32-wide boxes leave a quarter of theirs idle on
+// 100 x 50 x 70.  Bound by the latency of its scattered loads, hence the cap on
+// registers above; 100 x 50 x 70, moment-space collision: 25.1 us against 33.4 us
+// in 32 x 4 x 2 boxes.
+// The FP32 D3Q19 moment-space form sums its moments from a first read of the
+// populations and reads them again (from L1) for the collision, as the staged
+// kernels do from shared memory, instead of holding 36 of them beside the
+// stress moments (28.4 us).  The single-relaxation-time form is faster
+// with the populations in registers (27.4 against 30.3 us).
+template <class PT, class L, int NCOMP, bool STREAM, int COLL>
+__global__ void __launch_bounds__(128, (reg_blocks<PT, L, COLL>())) k_lattice(StepBufs b, StepParams p, int rev) {
+    const int i = tile_index(blockIdx.x, gridDim.x, rev) * 128 + threadIdx.x;
+    // densities, feedback stress and velocity are shared with the preceding pass
+    pdl_wait();
+    const long long N = p.N;
+    if (i >= N) return;
+    const int row = (int)((unsigned)i / (unsigned)p.nx), x = i - row * p.nx;
+    const int z = (int)((unsigned)row / (unsigned)p.ny), y = row - z * p.ny;
+    if constexpr (STREAM && L::D == 3 && COLL == 1 && sizeof(PT) == 4) {
+        const PT* fi = static_cast<const PT*>(b.fin) + i;
+        NodeGather<L, NCOMP> g;
+        node_gather<L, NCOMP>(b, p, x, y, z, true, g);
+        node_collide<PT, L, NCOMP, COLL>(
+            b, p, g, [&](int s, int a) { return pop_load(fi + (s * (L::Q - 1) + a - 1) * N); },
+            [&](int s, int a) { return pop_again(fi + (s * (L::Q - 1) + a - 1) * N); });
+        return;
+    }
 
     // moments (same summation order as k_moments)
     float f[NCOMP][L::Q];
@@ -571,68 +679,8 @@ __global__ void __launch_bounds__(128) k_lattice(StepBufs b, StepParams p, int r
         }
         return;
     }
+    pdl_trigger();
     collide_stream<PT, L, NCOMP, COLL>(b, p, nb, st, qloc, pif, [&](int s, int a) { return f[s][a]; });
-}
-
-// --- TMA-staged variant --------------------------------------------------------
-
-// Threads per SM the register budget of the staged lattice kernel is sized
-// for (1024: 64 registers per thread).
-#ifndef VEFD_LATTICE_THREADS_PER_SM
-#define VEFD_LATTICE_THREADS_PER_SM 1024
-#endif
-
-// Node work of the staged kernels, split around the wait for the staged
-// populations: gather (neighbour densities and feedback stress, overlapping
-// the copy), then moments, local state and collision from shared memory.
-template <class L, int NCOMP>
-struct NodeGather {
-    float dr[NCOMP];
-    float acc[2][3], Fp[3], qloc[L::NQ];
-    Nbr nb;
-};
-
-template <class L, int NCOMP>
-__device__ __forceinline__ void node_gather(const StepBufs& b, const StepParams& p, int x, int y, int z, bool active,
-                                            NodeGather<L, NCOMP>& g) {
-    g.nb = make_nbr(active ? x : 0, active ? y : 0, active ? z : 0, p);
-    if (!active) return;
-    // the node's own deviations come from the density buffer (bit-identical to
-    // the sum of the staged populations)
-    dens_ldg<NCOMP>(b.drho, g.nb.i, g.dr);
-    neighbour_forces<L, NCOMP>(b, p, g.nb, g.acc, g.Fp, g.qloc);
-}
-
-template <class PT, class L, int NCOMP, int T, int COLL, bool EDGE = true, bool PARTS = false>
-__device__ __forceinline__ void node_collide(const StepBufs& b, const StepParams& p, const PT* sf, int t,
-                                             const NodeGather<L, NCOMP>& g, PT* own = nullptr,
-                                             float* rest_out = nullptr) {
-    const long long N = p.N;
-    const int i = g.nb.i;
-    float jx = 0.0f, jy = 0.0f, jz = 0.0f;
-    float pif[NCOMP][6];
-#pragma unroll
-    for (int s = 0; s < NCOMP; ++s) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) pif[s][k] = 0.0f;
-#pragma unroll
-        for (int a = 1; a < L::Q; ++a) {
-            const float fa = pop_get(sf[(s * (L::Q - 1) + a - 1) * T + t]);
-            if (L::cx(a)) jx += L::cx(a) * fa;
-            if (L::cy(a)) jy += L::cy(a) * fa;
-            if (L::cz(a)) jz += L::cz(a) * fa;
-            if (COLL == 1) pi_add<L>(pif[s], a, fa);
-        }
-    }
-    Local<NCOMP> st;
-    local_state<L, NCOMP>(p, g.dr, jx, jy, jz, g.acc, g.Fp, st, b.status);
-    b.u[i] = st.ux;
-    b.u[N + i] = st.uy;
-    if (L::D == 3) b.u[2 * N + i] = st.uz;
-    // volatile reads keep the populations in shared memory instead of registers
-    collide_stream<PT, L, NCOMP, COLL, EDGE, PARTS>(
-        b, p, g.nb, st, g.qloc, pif, [&](int s, int a) { return pop_smem(sf, (s * (L::Q - 1) + a - 1) * T + t); },
-        own, T, rest_out);
 }
 
 // Partial densities of time n+1 from one staged D3Q19 tile (BX, BY, BZ >= 2),
@@ -1277,17 +1325,17 @@ cudaError_t launch_lattice_coll(int lattice, int ncomp, const StepParams& p, con
         return e;
     }
     if (parts.part) return cudaErrorInvalidValue;  // partial densities need the staged kernel
-    dim3 blk(32, 4, 1), grd = node_grid(p);
+    const unsigned nblk = (unsigned)((p.N + 127) / 128);
+    cudaError_t e = cudaSuccess;
     VEFD_WITH_PT(p.prec, {
-        if (lattice == 1) {
-            if (ncomp == 2) k_lattice<PT, D3Q19, 2, true, COLL><<<grd, blk, 0, s>>>(b, p, rev);
-            else k_lattice<PT, D3Q19, 1, true, COLL><<<grd, blk, 0, s>>>(b, p, rev);
-        } else {
-            if (ncomp == 2) k_lattice<PT, D2Q9, 2, true, COLL><<<grd, blk, 0, s>>>(b, p, rev);
-            else k_lattice<PT, D2Q9, 1, true, COLL><<<grd, blk, 0, s>>>(b, p, rev);
-        }
+        if (lattice == 1)
+            e = launch_pdl(p.pdl != 0, ncomp == 2 ? k_lattice<PT, D3Q19, 2, true, COLL> : k_lattice<PT, D3Q19, 1, true, COLL>,
+                           dim3(nblk), dim3(128), 0, s, b, p, rev);
+        else
+            e = launch_pdl(p.pdl != 0, ncomp == 2 ? k_lattice<PT, D2Q9, 2, true, COLL> : k_lattice<PT, D2Q9, 1, true, COLL>,
+                           dim3(nblk), dim3(128), 0, s, b, p, rev);
     });
-    return cudaGetLastError();
+    return e;
 }
 
 using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,

@@ -139,7 +139,7 @@ cudaError_t launch_lattice(int lattice, int ncomp, bool stream_pops, const StepP
     }
     if (parts.part) return cudaErrorInvalidValue;
     // macroscopic pass (moments, forces, velocity; no streaming)
-    dim3 blk(32, 4, 1), grd = node_grid(p);
+    const dim3 blk(128), grd((unsigned)((p.N + 127) / 128));
     VEFD_WITH_PT(p.prec, {
         if (lattice == 1) {
             if (ncomp == 2) k_lattice<PT, D3Q19, 2, false, 0><<<grd, blk, 0, s>>>(b, p, rev);

@@ -58,10 +58,10 @@ struct vefd_ctx {
     std::string err;
     // TMA descriptors of the two population buffers (when the shape allows)
     alignas(64) CUtensorMap tmap[2];       // lattice kernel: box = the selected staged tile
-    alignas(64) CUtensorMap tmap_post[2];  // densities/FD pass (3-D tile variant): box 32x4x2 or 32x8x1
+    alignas(64) CUtensorMap tmap_box[2];   // box of tile 0 (the ensembles' lattice launches)
     bool tma_ok = false;
     int lat_tile = 0;                      // staged tile shape of the lattice kernel (lattice_tile_shape)
-    int post_mode = 2;                     // 0 column march with fused densities, 1 3-D tiles, 2 separate z-march pass
+    int post_mode = 2;                     // 0 column march with fused densities, 1 runs of nodes, 2 separate z-march pass
     // tensor maps with a 32 x 8 x 1 box for the z-marching densities/FD pass
     alignas(64) CUtensorMap tmap_zm[2];
     bool zm_ok = false;
@@ -231,9 +231,8 @@ void build_tensor_maps(vefd_ctx* c) {
     c->fused_ok = false;
     c->parts_ok = false;
     if (getenv("VEFD_NO_TMA") || !pop_tile_eligible(lat, prec, nx, ny, nz, 0)) return;
-    // the densities/FD pass keeps the default tile
-    if (!(make_pop_tensor_map(lat, nc, prec, nx, ny, nz, c->f[0], &c->tmap_post[0]) &&
-          make_pop_tensor_map(lat, nc, prec, nx, ny, nz, c->f[1], &c->tmap_post[1])))
+    if (!(make_pop_tensor_map(lat, nc, prec, nx, ny, nz, c->f[0], &c->tmap_box[0]) &&
+          make_pop_tensor_map(lat, nc, prec, nx, ny, nz, c->f[1], &c->tmap_box[1])))
         return;
     int tile = pop_tile_eligible(lat, prec, nx, ny, nz, c->lat_tile) ? c->lat_tile : 0;
     c->lat_tile = tile;
@@ -360,6 +359,43 @@ uint64_t splitmix64(uint64_t seed, uint64_t i) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
 }
+
+// Whether the lattice kernel runs in staged boxes (else in runs of 128
+// consecutive nodes).  A tile chosen by the caller and the partial densities
+// keep their boxes; tile 0 does where its boxes are the faster form:
+// - D2Q9: from 2^18 nodes (1024 x 512 13.5 against 14.4 us; a step of 512 x 256
+//   6.8 against 6.7, of 200 x 100 4.1 against 3.8, of 64 x 32 3.8 against 3.5).
+// - D3Q19, single relaxation time: where the lattice fills three quarters of
+//   the boxes' nodes.  A box node costs 0.8 of a run's: 100 x 50 x 70 (fill 0.75)
+//   27.5 us both, 132 x 70 x 100 (0.80) 63.0 against 67.7, 68 x 36 x 50 (0.71)
+//   14.4 against 13.6.
+// - D3Q19, moment-space collision: 16-bit storage always (256 x 128 x 64 108
+//   against 112 us, 116 x 50 x 70 26.7 and 27.1), FP32 never (64^3 20.7 us in
+//   boxes, 19.7 in runs; 128 x 64 x 128 68.4 and 65.7, 132 x 70 x 100 73.2 and
+//   59.8).
+bool lattice_boxes(const vefd_ctx* c) {
+    if (!c->tma_ok) return false;
+    if (c->lat_tile != 0 || c->parts_ok) return true;
+    int bx, by, bz;
+    lattice_tile_shape(c->cfg.lattice, 0, &bx, &by, &bz);
+    const long long boxes = (long long)((c->cfg.nx + bx - 1) / bx) * ((c->cfg.ny + by - 1) / by) *
+                            ((c->cfg.nz + bz - 1) / bz);
+    const double fill = (double)c->N / ((double)boxes * bx * by * bz);
+    if (c->D == 2) return c->N >= (1 << 18) && fill >= 0.75;
+    if (c->collision == 1) return c->cfg.precision != 0;
+    return fill >= 0.75;
+}
+
+// Whether the densities/FENE-P pass marches columns along z (else runs of 128
+// consecutive nodes).  The march reads every stencil value 1.3 times instead of
+// 7, which pays once the pass is bound by memory; below, its segments are short
+// and its blocks few.  Steps in us, runs / columns: 32^3 6.5 / 9.0, 64 x 32 x 32
+// 9.2 / 11.8, 64^3 25.5 / 26.1 (FP16 22.6 / 24.8), 128 x 64 x 64 56.6 / 58.7,
+// 128 x 64 x 128 112.9 / 113.5 (FP16 95.2 / 96.4), 160 x 72 x 128 160.6 / 160.3,
+// 224 x 104 x 128 316 / 303 (FP16 269 / 263).  (The slab graph and the
+// batched ensembles march columns at every size.)
+constexpr long long kRunsMaxNodes = 1 << 20;
+bool post_columns(const vefd_ctx* c) { return c->zm_ok && (c->parts_ok || c->N > kRunsMaxNodes); }
 
 // The pipelined y-slab split applies for K slabs: staged lattice tiles (not
 // the persistent forms) with the separate z-marching pass, D3Q19, and rows
@@ -971,19 +1007,16 @@ static vefd_status step_eager(vefd_ctx* c, int64_t nsteps) {
             // populations n -> n+1, velocity of time n
             ProfScope ps(c, 1);
             VEFD_CUDA(c, launch_lattice(c->cfg.lattice, c->cfg.ncomp, true, p, b, c->stream,
-                                        c->tma_ok ? (const void*)&c->tmap[c->cur] : nullptr, lat_rev, c->lat_tile,
+                                        lattice_boxes(c) ? (const void*)&c->tmap[c->cur] : nullptr, lat_rev, c->lat_tile,
                                         parts_of(c)));
         }
         {
             // densities of time n+1 (they only depend on the new populations)
             // and the conformation update n -> n+1 (it only needs u^n and C^n)
             ProfScope ps(c, 2);
-            if (c->zm_ok)
+            if (post_columns(c))
                 VEFD_CUDA(c, launch_post_zm(c->cfg.ncomp, c->fd_on != 0, p, b, &c->tmap_zm[1 - c->cur], c->stream,
                                             post_rev, parts_of(c)));
-            else if (c->tma_ok)
-                VEFD_CUDA(c, launch_post_tma(c->cfg.lattice, c->cfg.ncomp, c->fd_on != 0, p, b, &c->tmap_post[1 - c->cur],
-                                             c->stream, post_rev));
             else
                 VEFD_CUDA(c, launch_post(c->cfg.lattice, c->cfg.ncomp, c->fd_on != 0, p, b, c->f[1 - c->cur],
                                          c->stream, post_rev));
@@ -1556,7 +1589,7 @@ vefd_status ens_build_table(vefd_ensemble* e) {
         M.p = params_of(m);
         M.cur0 = m->cur;
         for (int j = 0; j < 2; ++j) {
-            M.tm_lat[j] = e->tile == 1 ? m->tmap_zm[j] : m->tmap_post[j];  // box of the lattice tile
+            M.tm_lat[j] = e->tile == 1 ? m->tmap_zm[j] : m->tmap_box[j];  // box of the lattice tile
             M.tm_post[j] = m->tmap_zm[j];                                    // box 32 x 8 x 1
         }
         for (int par = 0; par < 2; ++par) {

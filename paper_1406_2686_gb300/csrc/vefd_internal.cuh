@@ -136,6 +136,23 @@ __device__ __forceinline__ __half pop_put<__half>(float v) { return __float2half
 template <>
 __device__ __forceinline__ __nv_bfloat16 pop_put<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 
+// second read of a population (kept from being merged with the first)
+__device__ __forceinline__ float pop_again(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float pop_again(const __half* p) {
+    unsigned short v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __half2float(__ushort_as_half(v));
+}
+__device__ __forceinline__ float pop_again(const __nv_bfloat16* p) {
+    unsigned short v;
+    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __bfloat162float(__ushort_as_bfloat16(v));
+}
+
 // volatile shared-memory read of a staged population (keeps it out of registers)
 __device__ __forceinline__ float pop_smem(const float* base, int idx) {
     return static_cast<const volatile float*>(base)[idx];
@@ -408,10 +425,6 @@ void lattice_tile_shape(int lattice, int tile, int* bx, int* by, int* bz);
 // stress of the new time level into b.Q.
 cudaError_t launch_post(int lattice, int ncomp, bool fd, const StepParams& p, const StepBufs& b,
                         const void* fnew, cudaStream_t s, int rev);
-// With a tensor map of `fnew` (TMA-eligible shapes), the same pass stages the
-// tile's populations with one bulk copy while the stencil loads are in flight.
-cudaError_t launch_post_tma(int lattice, int ncomp, bool fd, const StepParams& p, const StepBufs& b,
-                            const void* tensor_map_fnew, cudaStream_t s, int rev);
 // D3Q19 z-marching variant of the pass (needs NX % 32 == 0 and NY % 8 == 0 and a
 // tensor map of `fnew` with box 32 x 8 x 1 x P).
 bool post_zm_eligible(int lattice, int nx, int ny);
