@@ -344,8 +344,8 @@ vefd_status vefd_get_step_graph(vefd_ctx *ctx, int *slabs, int *chunk, int *acti
  * configurations together: `chunk` steps of all members are captured once as
  * a CUDA graph and replayed, either as two batched launches per step over the
  * tiles of all members (vefd_ensemble_set_batched) or with every member's
- * step as one graph branch, so small lattices fill the GPU together and pay
- * no per-launch host cost.  Members stay
+ * steps as one graph branch, the branches in sets whose state stays in L2, so
+ * small lattices fill the GPU together and pay no per-launch host cost.  Members stay
  * ordinary contexts (read, diagnose, checkpoint them as usual, between
  * ensemble calls); the ensemble does not own them and must be destroyed
  * before they are. */
@@ -367,7 +367,9 @@ vefd_status vefd_ensemble_create(vefd_ctx *const *members, int n, void *stream, 
  * member is not initialised, VEFD_ERR_CUDA on capture or launch errors
  * (see vefd_ensemble_last_error). */
 vefd_status vefd_ensemble_step(vefd_ensemble *ens, int64_t nsteps, int64_t chunk);
-/* Batched launches (default on): when every member is D3Q19 with the same
+/* Batched launches (default on; used for members of fewer than 2^14 or more
+ * than 2^19 nodes on average, or once a z-segment, group count or lattice tile
+ * is set): when every member is D3Q19 with the same
  * component count, storage type, collision operator, FENE-P switch and
  * programmatic-launch setting, and each takes the staged lattice kernel and
  * the separate z-marching densities/FENE-P pass (NX % 32 == 0, NY % 8 == 0,

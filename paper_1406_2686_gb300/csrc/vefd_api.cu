@@ -1476,7 +1476,8 @@ struct vefd_ensemble {
     cudaStream_t user = nullptr;       // caller's stream
     cudaStream_t main = nullptr;       // capture origin and graph launch stream
     cudaEvent_t fork = nullptr, done = nullptr;
-    int64_t chunk = 0;                 // steps per graph launch
+    int64_t chunk = 0;                 // the caller's steps per graph launch
+    int64_t span = 0;                  // steps of the captured graph (a divisor of chunk)
     cudaGraphExec_t exec = nullptr;
     std::vector<std::vector<double>> key;  // member state the graph was captured for
     std::string err;
@@ -1736,7 +1737,68 @@ vefd_status ens_eager(vefd_ensemble* e, int64_t n) {
     return VEFD_OK;
 }
 
-// Captures `chunk` steps of every member, one branch each, into e->exec.
+// Bytes of device memory a step of the member touches: both population
+// buffers, rest populations, densities, velocity, both conformation buffers,
+// the AB2 history and the stress.
+long long ens_step_bytes(const vefd_ctx* m) {
+    const long long pops = 2LL * m->cfg.ncomp * (m->Q - 1) * m->psize;
+    const long long words = m->cfg.ncomp + 2 + 3 + 3 * m->NC + (m->D == 3 ? 6 : 3);
+    return m->N * (pops + 4 * words);
+}
+
+// Members whose steps run side by side in the branch form, as consecutive
+// sets of `order` (the members by falling size, so that a set's members finish
+// together): two at least, and as many as fit kEnsSetBytes, so that a set's
+// whole state stays in L2 (129 MB) from step to step while its kernels cover
+// each other's launches and tails.  Steps of all members in us, all side by
+// side / batched launches / sets: 16 of 32^3 55.7 / 58.2 / 45.8, 16 of 64 x 32 x 32
+// 111 / 115 / 86.5, 16 of 64 x 64 x 32 217 / 222 / 171, FP16 - / 203 / 158, 8 of 64^3
+// FP16 186 / 201 / 174, 20 of mixed sizes (49k to 743k nodes) 501 / 507 / 474.
+// With 134 MB: 45.3, 94.1, 171, 176, 174 and 478.
+constexpr long long kEnsSetBytes = 96LL << 20;
+void ens_sets(const vefd_ensemble* e, std::vector<int>* order, std::vector<int>* first) {
+    const int n = (int)e->members.size();
+    order->resize(n);
+    for (int k = 0; k < n; ++k) (*order)[k] = k;
+    std::stable_sort(order->begin(), order->end(), [&](int a, int b) {
+        return ens_step_bytes(e->members[a]) > ens_step_bytes(e->members[b]);
+    });
+    first->assign(1, 0);
+    long long bytes = 0;
+    for (int k = 0; k < n; ++k) {
+        const long long add = ens_step_bytes(e->members[(*order)[k]]);
+        if (k - first->back() >= 2 && bytes + add > kEnsSetBytes) {
+            first->push_back(k);
+            bytes = 0;
+        }
+        bytes += add;
+    }
+    first->push_back(n);
+}
+
+// Whether the branch form is taken although the members admit batched
+// launches: their mean size is 2^14 to 2^19 nodes and nothing was set.  Smaller
+// ones are bound by their launches (64 of 32 x 16 x 16: 61 us batched, 49 in sets, but
+// four times the graph), larger ones gain nothing (2 of 128 x 64 x 128 217 / 219).
+bool ens_prefers_sets(const vefd_ensemble* e) {
+    long long total = 0;
+    for (const vefd_ctx* m : e->members) total += m->N;
+    const long long n = (long long)e->members.size();
+    return n >= 2 && e->post_seg == 0 && e->groups == 0 && e->tile == 0 && total >= n << 14 && total <= n << 19;
+}
+
+// Steps of one captured graph of the branch form: the largest even divisor of
+// the chunk from 8 to 16, else the chunk.  A set runs that many steps before
+// the next set's begin, enough to pay for loading its state; a longer graph
+// only takes longer to capture (20 boxes, 50 steps: first call 25.4 ms with
+// 10, 29.7 ms with 50; later ones 24.4 and 24.2 ms).
+int64_t ens_span(int64_t chunk) {
+    for (int64_t k = 16; k >= 8; k -= 2)
+        if (chunk % k == 0) return k;
+    return chunk;
+}
+
+// Captures `chunk` steps of every member, set after set, into e->exec.
 vefd_status ens_capture(vefd_ensemble* e, int64_t chunk) {
     const size_t n = e->members.size();
     std::vector<int> cur(n), ccur(n), hp(n);
@@ -1759,10 +1821,19 @@ vefd_status ens_capture(vefd_ensemble* e, int64_t chunk) {
         return ens_fail(e, VEFD_ERR_CUDA, "cannot begin capture");
     vefd_status st = VEFD_OK;
     std::string why;
-    cudaError_t ce = cudaEventRecord(e->fork, e->main);
-    for (size_t k = 0; k < n && ce == cudaSuccess && st == VEFD_OK; ++k) {
+    std::vector<int> order, first;
+    ens_sets(e, &order, &first);
+    cudaError_t ce = cudaSuccess;
+    for (size_t at = 0, set = 0; at < n && ce == cudaSuccess && st == VEFD_OK; ++at) {
+        if ((int)at == first[set]) {
+            // the origin stream has joined every branch of the set before
+            ++set;
+            ce = cudaEventRecord(e->fork, e->main);
+            for (int j = first[set - 1]; j < first[set] && ce == cudaSuccess; ++j)
+                ce = cudaStreamWaitEvent(e->branch[order[j]], e->fork, 0);
+        }
+        const size_t k = order[at];
         vefd_ctx* m = e->members[k];
-        ce = cudaStreamWaitEvent(e->branch[k], e->fork, 0);
         if (ce != cudaSuccess) break;
         m->stream = e->branch[k];
         m->prof_on = false;
@@ -1881,15 +1952,16 @@ vefd_status vefd_ensemble_step(vefd_ensemble* e, int64_t nsteps, int64_t chunk) 
         if (stale) {
             if (e->exec) cudaGraphExecDestroy(e->exec);
             e->exec = nullptr;
-            const vefd_status st =
-                e->batched_pref && ens_batchable(e) ? ens_capture_batched(e, chunk) : ens_capture(e, chunk);
+            const bool batched = e->batched_pref && ens_batchable(e) && !ens_prefers_sets(e);
+            e->span = batched ? chunk : ens_span(chunk);
+            const vefd_status st = batched ? ens_capture_batched(e, chunk) : ens_capture(e, e->span);
             if (st != VEFD_OK) return st;
             e->chunk = chunk;
             e->key.resize(e->members.size());
             for (size_t k = 0; k < e->members.size(); ++k) e->key[k] = ens_key(e->members[k]);
         }
         if (ens_wait_inputs(e, e->main) != cudaSuccess) return ens_fail(e, VEFD_ERR_CUDA, "ordering after the inputs failed");
-        for (int64_t r = 0; r < full; ++r)
+        for (int64_t r = 0; r < full * (chunk / e->span); ++r)
             if (cudaGraphLaunch(e->exec, e->main) != cudaSuccess) return ens_fail(e, VEFD_ERR_CUDA, "graph launch failed");
         // an even chunk leaves every ping-pong parity where it was
         for (vefd_ctx* m : e->members) m->steps += full * chunk;

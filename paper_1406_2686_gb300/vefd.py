@@ -573,9 +573,10 @@ class Lattice:
 
 
 class Ensemble:
-    """Independent lattices stepped together as one replayed CUDA graph: two
-    batched launches per step over all members when they allow it, else one
-    concurrent branch per lattice.  Holds references to its members."""
+    """Independent lattices stepped together as one replayed CUDA graph: small
+    and very large ones by two batched launches per step over all members when
+    they allow it, else one branch per lattice, in sets of branches whose state
+    stays in L2.  Holds references to its members."""
 
     def __init__(self, lattices, stream=None):
         import torch
@@ -587,8 +588,8 @@ class Ensemble:
         vefd_ensemble_step(self.ens, n, chunk)
 
     def set_batched(self, on):
-        """One launch per kernel phase over all members (default), or one
-        graph branch per member."""
+        """One launch per kernel phase over all members where that is the
+        faster form (default), or always one graph branch per member."""
         vefd_ensemble_set_batched(self.ens, 1 if on else 0)
 
     @property

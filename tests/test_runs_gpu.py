@@ -39,3 +39,24 @@ def test_runs_give_the_bits_of_the_boxes(box, collision):
     tol = 2e-5 if collision == 1 and d3 else 0.0
     for a, b in zip(state(A), state(B)):
         assert np.isfinite(a).all() and np.abs(a - b).max() <= tol
+
+
+@pytest.mark.parametrize("chunk", [16, 22, 50])
+def test_ensemble_sets_give_the_members_bits(chunk):
+    """Members of 2^14 nodes and more step in sets that stay in L2: uneven
+    sizes and several sets, graphs shorter than the chunk (10 of 50 steps), equal
+    to it (16) and without a divisor (22), and a remainder of eager steps."""
+    from paper_1406_2686_gb300 import vefd
+    sizes = [(64, 32, 32), (32, 40, 35), (96, 32, 32), (64, 64, 33), (64, 32, 32), (32, 32, 16)]
+    boxes = [dict(COMMON, lattice=1, nx=x, ny=y, nz=z, ncomp=2, walls=k % 2, u_wall=0.03 * (k % 2))
+             for k, (x, y, z) in enumerate(sizes)]
+    ens, alone = [[make(b, seed=20 + k) for k, b in enumerate(boxes)] for _ in range(2)]
+    E = vefd.Ensemble(ens)
+    for n in (1 + 2 * chunk, chunk + 3):
+        E.step(n, chunk=chunk)
+        assert not E.batched
+        for L in alone:
+            L.step(n)
+    for a, b in zip(ens, alone):
+        assert a.steps_done == b.steps_done
+        assert all(np.array_equal(x, y) for x, y in zip(state(a), state(b)))
