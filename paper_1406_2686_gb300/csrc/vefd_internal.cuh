@@ -420,6 +420,12 @@ cudaError_t launch_post_batch(int ncomp, int prec, bool fd, const EnsMember* mem
 // Staged tile shapes of the lattice kernel: tile 0..2 ->
 // D3Q19 32x4x2, 32x2x4, 32x8x1; D2Q9 32x8x1, 32x4x1, 32x16x1.
 void lattice_tile_shape(int lattice, int tile, int* bx, int* by, int* bz);
+// `nsteps` >= 1 steady steps (current densities, AB2 history when fd) of a D2Q9
+// lattice of up to kSmallMaxNodes nodes in one launch (k_small); the state ends
+// in the buffers that as many single steps leave it in.  cudaErrorNotSupported
+// where the device cannot run the cluster.
+constexpr int kSmallBlocks = 16, kSmallMaxThreads = 512, kSmallMaxNodes = kSmallBlocks * kSmallMaxThreads;
+cudaError_t launch_small(int ncomp, bool fd, const StepParams& p, const StepBufs& b, int nsteps, cudaStream_t s);
 // Densities of the populations `fnew` into b.drho, when fd the FENE-P update
 // b.Cin -> b.Cout with the AB2 history b.R and velocity b.u, and the feedback
 // stress of the new time level into b.Q.

@@ -58,5 +58,33 @@ def test_ensemble_sets_give_the_members_bits(chunk):
         for L in alone:
             L.step(n)
     for a, b in zip(ens, alone):
-        assert a.steps_done == b.steps_done
+        assert vefd.vefd_steps_done(a.ctx) == vefd.vefd_steps_done(b.ctx)
         assert all(np.array_equal(x, y) for x, y in zip(state(a), state(b)))
+
+
+SMALL = [
+    dict(nx=64, ny=32, ncomp=1, walls=1, u_wall=0.03, G=0.0),               # 16 blocks of 128 nodes
+    dict(nx=13, ny=11, ncomp=2, walls=0),                                   # some blocks have no node
+    dict(nx=35, ny=40, ncomp=2, walls=1, u_wall=0.03, precision=1),         # the last block is partial
+    dict(nx=128, ny=64, ncomp=2, walls=1, u_wall=0.03, coupling=1),         # the largest
+    dict(nx=91, ny=90, ncomp=1, walls=0, precision=2, G=0.0, fext=(1e-5, 2e-5, 0.0)),
+]
+
+
+@pytest.mark.parametrize("collision", [0, 1])
+@pytest.mark.parametrize("box", range(len(SMALL)))
+def test_many_steps_in_one_launch_give_the_bits_of_single_steps(box, collision):
+    from paper_1406_2686_gb300 import vefd
+    A, B = (make(dict(COMMON, lattice=0, **SMALL[box]), seed=40 + box) for _ in range(2))
+    B.set_step_graph(0)  # launch pairs
+    for L in (A, B):
+        L.set_collision(collision)
+        L.set_conformation_update(box % 2)
+        L.set_body_force(0.0, 0.0, 0.0)
+    for n in (9, 1, 4, 6, 1030):  # with the Euler start; odd counts; two launches
+        A.step(n)
+        B.step(n)
+    assert vefd.vefd_steps_done(A.ctx) == vefd.vefd_steps_done(B.ctx)
+    for f in (vefd.POPS, vefd.C, vefd.RPREV, vefd.U, vefd.PHI, vefd.RHO_A):
+        a, b = A.read(f), B.read(f)
+        assert np.isfinite(a).all() and np.array_equal(a, b)
