@@ -43,6 +43,7 @@ namespace {
 constexpr int kTaps = 27;
 constexpr int kConvThreads = 256;       // warps 0-3 epilogue, 4 and 6 matrix operations, 5 weights, 7 halo copies
 constexpr int kBStages = 4;             // ring of weight chunks
+constexpr int kTapPlanes = 3;           // groups of halo planes that land one after the other
 constexpr int kMaxPairs = 512;          // K = 16 steps of a channel block
 constexpr unsigned kSmemMax = 217u * 1024u;
 
@@ -203,11 +204,11 @@ __device__ __forceinline__ uint4 pack8(const float* f) {
 // its own copies or matrix operations before tensor memory is freed.
 __global__ void __launch_bounds__(kConvThreads, 2)
     k_conv(const __grid_constant__ CUtensorMap tm0, const __grid_constant__ CUtensorMap tm1,
-           const __grid_constant__ Halo h, const __grid_constant__ Entries ent, const uint4* __restrict__ Wk, int Np, int bn,
-           int nbuf, int nset, int cols, int chunk, float* __restrict__ Y, uint4* __restrict__ Yb, int Do, int Ho,
+           const __grid_constant__ CUtensorMap tmw, const __grid_constant__ Halo h, const __grid_constant__ Entries ent, const uint4* __restrict__ Wk, int Np, int bn,
+           int nbuf, int nset, int cols, int chunk, int groups, float* __restrict__ Y, uint4* __restrict__ Yb, int Do, int Ho,
            int Wo, const float* __restrict__ bias, int N, int relu, int vec, unsigned* __restrict__ status) {
     extern __shared__ __align__(128) unsigned char dsm[];
-    __shared__ __align__(8) unsigned long long afull[2], aempty[2], bfull[kBStages], bempty[kBStages], acc_full[2],
+    __shared__ __align__(8) unsigned long long afull[2][kTapPlanes], aempty[2], bfull[kBStages], bempty[kBStages], acc_full[2],
         acc_empty[2], drain[2];
     __shared__ __align__(16) uint2 pairs[kMaxPairs + 2];
     __shared__ unsigned tmem_base;
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     const int ntn = (Np + bn - 1) / bn, nitems = h.ntiles * ntn;
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
-            mbar_init_n(smem_addr(&afull[s]), 1);
+            for (int g = 0; g < kTapPlanes; ++g) mbar_init_n(smem_addr(&afull[s][g]), 1);
             mbar_init_n(smem_addr(&aempty[s]), 2);
             mbar_init_n(smem_addr(&acc_full[s]), 2);
             mbar_init_n(smem_addr(&acc_empty[s]), 4);
@@ -301,7 +302,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
     } else if (warp == 5) {
         int ib = 0;
         for (int t = blockIdx.x; t < nitems && !failed; t += gridDim.x) {
-            const int n0 = (t % ntn) * bn, bw = min(bn, Np - n0);
+            const int n0 = (t % ntn) * bn;
             for (int q = 0; q < nchunk * h.nblk; ++q, ++ib) {
                 const int sb = ib % kBStages, blk = q / nchunk, c = q % nchunk;
                 if (ib >= kBStages && !mbar_wait(smem_addr(&bempty[sb]), (unsigned)((ib / kBStages - 1) & 1))) failed = true;
@@ -309,17 +310,20 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                     failed = true;
                     break;
                 }
-                const int n = 2 * min(chunk, ent.npairs - c * chunk);  // pieces
                 const unsigned bb = smem_addr(&bfull[sb]), dst = b_base + (unsigned)sb * b_bytes;
-                const uint4* src = Wk + ((long long)blk * ent.npairs + c * chunk) * 2 * Np + n0;
-                if (lane == 0) mbar_expect(bb, (unsigned)(n * bw) * 16u);
-                __syncwarp();
-                if (bn == Np) {
-                    if (lane == 0) bulk_load(dst, src, (unsigned)(n * bn) * 16u, bb);
-                } else {
-                    for (int k = lane; k < n; k += 32)
-                        bulk_load(dst + (unsigned)(k * bn) * 16u, src + (long long)k * Np, bw * 16u, bb);
+                const long long piece = ((long long)blk * ent.npairs + c * chunk) * 2;
+                if (lane == 0) {
+                    if (bn == Np) {
+                        const unsigned bytes = 2u * (unsigned)min(chunk, ent.npairs - c * chunk) * (unsigned)bn * 16u;
+                        mbar_expect(bb, bytes);
+                        bulk_load(dst, Wk + piece * Np, bytes, bb);
+                    } else {
+                        // one box of chunk pieces x bn columns (zeros beyond the arrays count as copied)
+                        mbar_expect(bb, b_bytes);
+                        tma_load_2d(dst, &tmw, n0 * 2, (int)piece, bb);
+                    }
                 }
+                __syncwarp();
             }
         }
         if (failed) *abortp = 1;
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         for (int q = ib > kBStages ? ib - kBStages : 0; q < ib; ++q)
             mbar_wait(smem_addr(&bfull[q % kBStages]), (unsigned)((q / kBStages) & 1));
     } else if (warp == 7) {
-        const unsigned tx = (unsigned)(h.slabs * h.s) * (unsigned)(h.hx * h.hy * h.hz) * 16u;
+        const unsigned tx = (unsigned)(h.slabs * h.s) * (unsigned)(h.hx * h.hy) * 16u;  // of one plane
         int ia = 0;
         for (int t = blockIdx.x; t < nitems && !failed; t += gridDim.x) {
             const TileAt a = tile_at(h, t / ntn);
@@ -338,19 +342,28 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                     failed = true;
                     break;
                 }
-                if (lane == 0) mbar_expect(smem_addr(&afull[s]), tx);
-                __syncwarp();
-                for (int p = lane; p < h.slabs; p += 32) {
-                    // slab p: piece p of the block, or with the copy in front (odd Cb) piece p - 1
-                    const int c = h.slabs == h.Cb ? blk * h.Cb + p : (p == 0 ? h.Cb : p) - 1;
-                    stage_slab(h, &tm0, &tm1, a, a.z * h.s + h.lo, base + (unsigned)s * a_bytes + (unsigned)p * h.pitch_slab,
-                               c * 8, smem_addr(&afull[s]));
+                for (int g = 0; g < groups; ++g) {
+                    const unsigned bar = smem_addr(&afull[s][g]);
+                    const int z0 = g == 0 ? 0 : h.hz - groups + g, nz = g == 0 ? h.hz - groups + 1 : 1;
+                    if (lane == 0) mbar_expect(bar, tx * (unsigned)nz);
+                    __syncwarp();
+                    const int boxes = groups == 1 ? 1 : nz;  // a box is the whole halo or one plane
+                    for (int p = lane; p < h.slabs * boxes; p += 32) {
+                        // slab q: piece q of the block, or with the copy in front (odd Cb) piece q - 1
+                        const int q = p / boxes, z = z0 + p % boxes;
+                        const int c = h.slabs == h.Cb ? blk * h.Cb + q : (q == 0 ? h.Cb : q) - 1;
+                        stage_slab(h, &tm0, &tm1, a, a.z * h.s + h.lo + z,
+                                   base + (unsigned)s * a_bytes + (unsigned)q * h.pitch_slab + (unsigned)z * h.pitch_plane,
+                                   c * 8, bar);
+                    }
+                    __syncwarp();
                 }
             }
         }
         if (failed) *abortp = 1;
         // bounded: the copies in flight land before the block leaves
-        for (int q = ia > nbuf ? ia - nbuf : 0; q < ia; ++q) mbar_wait(smem_addr(&afull[q % nbuf]), (unsigned)((q / nbuf) & 1));
+        for (int q = ia > nbuf ? ia - nbuf : 0; q < ia; ++q)
+            for (int g = 0; g < groups; ++g) mbar_wait(smem_addr(&afull[q % nbuf][g]), (unsigned)((q / nbuf) & 1));
     } else {
         const unsigned me = warp == 6;  // this warp's accumulators: run * T + t odd or even
         const unsigned a_hi = ((unsigned)h.s * h.pitch_y >> 4) | (1u << 14);
@@ -365,14 +378,20 @@ __global__ void __launch_bounds__(kConvThreads, 2)
             tc_fence_after();
             for (int blk = 0; blk < h.nblk && !failed; ++blk, ++ia) {
                 const int s = ia % nbuf;
-                failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&afull[s]), (unsigned)((ia / nbuf) & 1)) || *abortp);
+                int landed = 0;  // plane groups waited for
                 const unsigned base16 = (base + (unsigned)s * a_bytes) >> 4;
                 for (int c = 0; c < nchunk && !failed; ++c, ++ib) {
                     const int sb = ib % kBStages;
                     failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&bfull[sb]), (unsigned)((ib / kBStages) & 1)) || *abortp);
                     if (failed) break;
-                    tc_fence_after();
                     const int k0 = c * chunk, k1 = min(k0 + chunk, ent.npairs);
+                    // the first step that reads tap plane g is 9 g Cb / 2
+                    while (landed < groups && 2 * k1 > 9 * landed * h.Cb && !failed) {
+                        failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&afull[s][landed]), (unsigned)((ia / nbuf) & 1)) || *abortp);
+                        ++landed;
+                    }
+                    if (failed) break;
+                    tc_fence_after();
                     const unsigned b_lo = ((b_base + (unsigned)sb * b_bytes) >> 4) | ((unsigned)bn << 16);
                     const unsigned dset = tmem + (unsigned)set * set_cols;
                     if (ent.nrun > 1) issue_runs(pairs, k0, k1, me, base16, a_hi, b_lo, bn, dset, idesc, blk > 0);
@@ -703,9 +722,10 @@ void channel_blocks(int kind, int s, int C8, int* nblk, int* Cb) {
     *Cb = *nblk == 1 ? C8 : round_up((C8 + *nblk - 1) / *nblk, 2);
 }
 
-// Strides of the staged halo: boxes land 128-byte aligned.
-void set_pitches(Halo& h) {
+// Strides of the staged halo: boxes (all planes, or one each) land 128-byte aligned.
+void set_pitches(Halo& h, bool plane_boxes = false) {
     h.pitch_y = h.hx * 16, h.pitch_plane = h.hy * h.pitch_y;
+    if (plane_boxes) h.pitch_plane = round_up(h.pitch_plane, 128);
     h.pitch_par = round_up(h.hz * h.pitch_plane, 128);
     h.pitch_slab = h.s * h.pitch_par;
 }
@@ -836,12 +856,25 @@ bool grid_map(CUtensorMap* out, const void* base, int B, int D, int H, int W, in
 }
 
 bool halo_maps(CUtensorMap* tm0, CUtensorMap* tm1, const void* A, const Halo& h, int bz) {
-    return grid_map(tm0, A, h.B, h.D, h.H, h.W, h.C8, h.s, 0, h.hx, h.hy, bz) &&
-           grid_map(tm1, A, h.B, h.D, h.H, h.W, h.C8, h.s, h.s - 1, h.hx, h.hy, bz);
+    if (!grid_map(tm0, A, h.B, h.D, h.H, h.W, h.C8, h.s, 0, h.hx, h.hy, bz)) return false;
+    *tm1 = *tm0;  // stride 1 has one tensor
+    return h.s == 1 || grid_map(tm1, A, h.B, h.D, h.H, h.W, h.C8, h.s, h.s - 1, h.hx, h.hy, bz);
+}
+
+// Tensor map of packed weights [piece][Np][8 BF16] in 8-byte elements, with
+// boxes of `pieces` pieces x bn columns.
+bool weight_map(CUtensorMap* out, const void* wk, long long npieces, int Np, int bn, int pieces) {
+    const EncodeTiled encode = tensor_map_encoder();
+    if (!encode) return false;
+    const cuuint64_t dims[2] = {(cuuint64_t)Np * 2, (cuuint64_t)npieces}, strides[1] = {(cuuint64_t)Np * 16};
+    const cuuint32_t box[2] = {(cuuint32_t)bn * 2, (cuuint32_t)pieces}, one[2] = {1, 1};
+    return encode(out, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, 2, const_cast<void*>(wk), dims, strides, box, one,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 struct ConvPlan {
-    int PY, T, bn, chunk, nbuf, nset, occ;
+    int PY, T, bn, chunk, nbuf, nset, occ, groups;
     unsigned smem;
     bool ok;
 };
@@ -853,7 +886,7 @@ struct ConvPlan {
 // accumulator, 450 a chunk of weights, and 1500 between the items of a block;
 // 6000 for launch and the first copies.  (Deep levels, a few hundred steps over
 // a few tiles, are a chain of steps and chunks; the fine ones fill the SMs.)
-ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, int nrun, int npairs) {
+ConvPlan search_plan(int kind, int B, int D, int H, int W, int C8, int s, int Np, int nrun, int npairs) {
     ConvPlan best{};
     double best_t = 0.0;
     for (int PY = 8; PY <= 16; PY += 8)
@@ -861,20 +894,29 @@ ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, 
             if (kind == 1 && T > 1) continue;
             const Halo h = halo_of(kind, B, D, H, W, C8, s, PY, T);
             if (!h.ntiles) continue;
+            Halo hp = h;  // staged plane by plane
+            set_pitches(hp, true);
             int last = 0;
             for (int nt = 1; nt <= (Np + 15) / 16; ++nt) {
                 const int bn = round_up((Np + nt - 1) / nt, 16), set = nrun * T * bn;
-                if (bn > 256 || set > 512 || bn == last) continue;
+                if (bn > (nt == 1 ? 256 : 128) || set > 512 || bn == last) continue;
                 last = bn;
                 for (int chunk = 2; chunk <= 32; chunk *= 2) {
-                    ConvPlan p{PY, T, bn, chunk, 2, set <= 256 ? 2 : 1, 1, 0, true};
-                    const unsigned a = h.slabs * h.pitch_slab, ring = kBStages * (unsigned)chunk * 2 * bn * 16;
-                    if (2 * a + ring > kSmemMax) p.nbuf = 1;
-                    p.smem = p.nbuf * a + ring;
-                    if (p.smem > kSmemMax) continue;
+                    ConvPlan p{PY, T, bn, chunk, 2, set <= 256 ? 2 : 1, 1, 1, 0, true};
+                    const unsigned ring = kBStages * (unsigned)chunk * 2 * bn * 16;
                     const int cols = acc_alloc(p.nset * set);
-                    p.occ = std::max(1, std::min(4, std::min((int)(kSmemMax / (p.smem + 5120)), 512 / cols)));
-                    const long long items = (long long)h.ntiles * ((Np + bn - 1) / bn), slots = (long long)sm_count() * p.occ;
+                    const long long items = (long long)h.ntiles * ((Np + bn - 1) / bn);
+                    auto fit = [&](const Halo& g) {
+                        const unsigned a = g.slabs * g.pitch_slab;
+                        p.nbuf = 2 * a + ring > kSmemMax ? 1 : 2;
+                        p.smem = p.nbuf * a + ring;
+                        p.occ = std::max(1, std::min(4, std::min((int)(kSmemMax / (p.smem + 5120)), 512 / cols)));
+                    };
+                    fit(hp);
+                    if (kind == 0 && p.smem <= kSmemMax && items <= (long long)sm_count() * p.occ) p.groups = kTapPlanes;
+                    else fit(h);
+                    if (p.smem > kSmemMax) continue;
+                    const long long slots = (long long)sm_count() * p.occ;
                     const double load = (double)h.nblk * (1.0 * h.hz * h.hy * h.hx * h.s * h.slabs + 1500.0);
                     const double steps = (double)npairs * h.nblk;
                     const double mma = steps * T * std::max(39.0, bn / 2.0);               // the SM's tensor core
@@ -894,6 +936,26 @@ ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, 
     return best;
 }
 
+// The search takes longer on the host than a small layer on the device, so
+// each thread keeps the plans of the last layer shapes it launched.
+ConvPlan plan_conv(int kind, int B, int D, int H, int W, int C8, int s, int Np, int nrun, int npairs) {
+    struct Slot {
+        int key[8];
+        ConvPlan plan;
+    };
+    constexpr int kSlots = 64;
+    static thread_local Slot slots[kSlots];  // plan.ok == false: empty
+    const int key[8] = {kind, B, D, H, W, C8, s, Np};
+    unsigned at = 0;
+    for (int v : key) at = (at * 31u + (unsigned)v) * 2654435761u;
+    Slot& q = slots[at >> 26];
+    if (!q.plan.ok || !std::equal(key, key + 8, q.key)) {
+        q.plan = search_plan(kind, B, D, H, W, C8, s, Np, nrun, npairs);
+        std::copy(key, key + 8, q.key);
+    }
+    return q.plan;
+}
+
 // kind as halo_of; N output channels, Y on the grid Do x Ho x Wo.
 cudaError_t launch_conv(int kind, const void* A, int B, int D, int H, int W, int C8, int s, const void* wk, int N, float* Y,
                         void* Yb, int Do, int Ho, int Wo, const float* bias, int relu, unsigned* status, cudaStream_t st) {
@@ -902,18 +964,20 @@ cudaError_t launch_conv(int kind, const void* A, int B, int D, int H, int W, int
     if (e.npairs > kMaxPairs) return cudaErrorInvalidValue;
     const ConvPlan p = plan_conv(kind, B, D, H, W, C8, s, Np, nrun, e.npairs);
     if (!p.ok) return cudaErrorInvalidValue;
-    const Halo h = halo_of(kind, B, D, H, W, C8, s, p.PY, p.T);
+    Halo h = halo_of(kind, B, D, H, W, C8, s, p.PY, p.T);
+    set_pitches(h, p.groups > 1);
     e = kind == 1 ? adjoint_entries(h) : conv_entries(h);
-    CUtensorMap tm0, tm1;
-    if (!halo_maps(&tm0, &tm1, A, h, h.hz)) return cudaErrorInvalidValue;
-    const cudaError_t err = cudaFuncSetAttribute(k_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
-    if (err != cudaSuccess) return err;
     const long long items = (long long)h.ntiles * ((Np + p.bn - 1) / p.bn);
     if (items > 0x3fffffffLL) return cudaErrorInvalidValue;
-    const int vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
     const int grid = (int)std::min<long long>(items, (long long)sm_count() * p.occ);
-    k_conv<<<grid, kConvThreads, p.smem, st>>>(tm0, tm1, h, e, (const uint4*)wk, Np, p.bn, p.nbuf, p.nset,
-                                               acc_alloc(p.nset * nrun * p.T * p.bn), p.chunk, Y, (uint4*)Yb, Do, Ho, Wo, bias, N, relu,
+    CUtensorMap tm0, tm1, tmw{};
+    if (!halo_maps(&tm0, &tm1, A, h, p.groups == 1 ? h.hz : 1)) return cudaErrorInvalidValue;
+    if (p.bn < Np && !weight_map(&tmw, wk, (long long)h.nblk * e.npairs * 2, Np, p.bn, p.chunk * 2)) return cudaErrorInvalidValue;
+    static const cudaError_t err = cudaFuncSetAttribute(k_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    if (err != cudaSuccess) return err;
+    const int vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
+    k_conv<<<grid, kConvThreads, p.smem, st>>>(tm0, tm1, tmw, h, e, (const uint4*)wk, Np, p.bn, p.nbuf, p.nset,
+                                               acc_alloc(p.nset * nrun * p.T * p.bn), p.chunk, p.groups, Y, (uint4*)Yb, Do, Ho, Wo, bias, N, relu,
                                                vec, status);
     return cudaGetLastError();
 }

@@ -129,6 +129,13 @@ __device__ __forceinline__ void tmem_ld16(unsigned addr, uint32_t v[16]) {
 }
 
 // Tiled bulk tensor copy of one 5-D box into shared memory (128-byte aligned), zero beyond the tensor.
+__device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* tm, int c0, int c1, unsigned bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+        "l"(reinterpret_cast<unsigned long long>(tm)), "r"(c0), "r"(c1), "r"(bar)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_5d(unsigned dst, const CUtensorMap* tm, int c0, int c1, int c2, int c3, int c4,
                                             unsigned bar) {
     asm volatile(

@@ -165,16 +165,16 @@ class Conv3d:
         B, D, H, W, C = x.shape
         assert C == self.cin and x.is_contiguous()
         xb = torch.empty(B * D * H * W, round8(C), dtype=torch.bfloat16, device="cuda")
-        return self._forward(x, xb, x.shape, None)
+        return self._forward(x, xb, x.shape, None, _stream())
 
-    def _forward(self, x, xb, shape, yb):
+    def _forward(self, x, xb, shape, yb, stream):
         """The layer on x, or on the BF16 copy xb alone (x None); yb receives the output's."""
         import torch
         B, D, H, W, C = shape
         y = torch.empty(self.out_shape(shape), device="cuda")
-        _check(L().vefd_nn_conv3d_forward(_p(x), B, D, H, W, C, self.stride, _p(self.wk), _p(self.b), self.cout,
-                                          int(self.relu), _p(xb), _p(y), _p(yb), _p(self.status), _stream()),
-               "conv3d_forward")
+        _check(L().vefd_nn_conv3d_forward(_p(x), B, D, H, W, C, self.stride, self.wk.data_ptr(), self.b.data_ptr(),
+                                          self.cout, int(self.relu), xb.data_ptr(), y.data_ptr(), _p(yb),
+                                          self.status.data_ptr(), stream), "conv3d_forward")
         self._saved = (shape, xb, y)
         return y
 
@@ -186,12 +186,12 @@ class Conv3d:
         dy = dy.reshape(y.shape).contiguous()
         if dy.data_ptr() % 16:
             dy = dy.clone()
-        lb, size = L(), (B, D, H, W, C, self.stride)
+        lb, size, stream = L(), (B, D, H, W, C, self.stride), _stream()
         scratch = torch.empty(lb.vefd_nn_conv3d_backward_scratch(*size, self.cout), device="cuda")
         dx = torch.empty(xshape, device="cuda")
         _check(lb.vefd_nn_conv3d_backward(_p(xb), _p(y), _p(dy), *size, _p(self.wd), self.cout, int(self.relu),
                                           _p(scratch), _p(self.dw), _p(self.db), int(accumulate), _p(dx),
-                                          _p(self.status), _stream()), "conv3d_backward")
+                                          _p(self.status), stream), "conv3d_backward")
         self._saved = None
         return dx
 
@@ -281,6 +281,7 @@ class UNet:
 
     def forward(self, x):
         import torch
+        stream = _stream()  # asking for it takes as long as a launch
 
         def grid(shape):
             return torch.empty(shape, dtype=torch.bfloat16, device="cuda")
@@ -290,7 +291,7 @@ class UNet:
             layer writes the copy that the next one reads."""
             for lay in layers:
                 yb = grid(lay.out_shape(shape)) if lay is not self.layers[-1] else None
-                x, xb, shape = None, yb, (y := lay._forward(x, xb, shape, yb)).shape
+                x, xb, shape = None, yb, (y := lay._forward(x, xb, shape, yb, stream)).shape
             return y, yb
 
         def up(layers, ub, sb):
@@ -298,7 +299,7 @@ class UNet:
             B, D, H, W, Cs = sb.shape
             shape = (B, D, H, W, ub.shape[-1] + Cs)
             xb = grid(shape)
-            _check(L().vefd_nn_up_concat(_p(ub), ub.shape[-1], _p(sb), Cs, B, D, H, W, _p(xb), _stream()), "up_concat")
+            _check(L().vefd_nn_up_concat(_p(ub), ub.shape[-1], _p(sb), Cs, B, D, H, W, _p(xb), stream), "up_concat")
             return run(layers, None, xb, shape)
 
         B, D, H, W, C = x.shape
