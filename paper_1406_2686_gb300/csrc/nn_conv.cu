@@ -186,6 +186,13 @@ __device__ __forceinline__ void issue_runs(const uint2* pairs, int k0, int k1, u
     }
 }
 
+// Wait of a whole warp.  A phase that is complete already, the common case in
+// front of a chunk, costs one poll; only a wait that is not looks at the abort flag.
+__device__ __forceinline__ bool warp_wait(unsigned bar, unsigned parity, volatile int* abortp) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity) && !*abortp);
+}
+
 __device__ __forceinline__ uint4 pack8(const float* f) {
     __nv_bfloat162 h[4];
 #pragma unroll
@@ -382,12 +389,12 @@ __global__ void __launch_bounds__(kConvThreads, 2)
                 const unsigned base16 = (base + (unsigned)s * a_bytes) >> 4;
                 for (int c = 0; c < nchunk && !failed; ++c, ++ib) {
                     const int sb = ib % kBStages;
-                    failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&bfull[sb]), (unsigned)((ib / kBStages) & 1)) || *abortp);
+                    failed = !warp_wait(smem_addr(&bfull[sb]), (unsigned)((ib / kBStages) & 1), abortp);
                     if (failed) break;
                     const int k0 = c * chunk, k1 = min(k0 + chunk, ent.npairs);
                     // the first step that reads tap plane g is 9 g Cb / 2
                     while (landed < groups && 2 * k1 > 9 * landed * h.Cb && !failed) {
-                        failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&afull[s][landed]), (unsigned)((ia / nbuf) & 1)) || *abortp);
+                        failed = !warp_wait(smem_addr(&afull[s][landed]), (unsigned)((ia / nbuf) & 1), abortp);
                         ++landed;
                     }
                     if (failed) break;
@@ -523,7 +530,7 @@ __global__ void __launch_bounds__(kConvThreads, 2)
         const unsigned ky = (unsigned)h.s * h.pitch_y;  // voxel groups: one tile row apart
         for (int it = 0; it < nt; ++it) {
             const int s = it % stages;
-            failed = __any_sync(0xffffffffu, !mbar_wait(smem_addr(&full[s]), (unsigned)((it / stages) & 1)) || *abortp);
+            failed = !warp_wait(smem_addr(&full[s]), (unsigned)((it / stages) & 1), abortp);
             if (failed) break;
             tc_fence_after();
             const unsigned sa = base + (unsigned)s * stage_bytes, sb = sa + a_bytes;
