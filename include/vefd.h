@@ -265,7 +265,8 @@ vefd_status vefd_set_kernel_config(vefd_ctx *ctx, int lattice_tile, int post_mod
  *   VEFD_SCHEDULE=b      bit 0 walks the lattice kernel's tiles, bit 1 the pass's
  *                        columns in reverse order (default 0);
  *   VEFD_ZM_SEGMENT=n    z-segment length of the column march (default: one wave);
- *   VEFD_SLAB_SEGMENT=n  z-segment of the step graph's slab passes (default 12);
+ *   VEFD_SLAB_SEGMENT=n  z-segment of the step graph's slab passes (default: 12 to 64
+ *                        planes, so that a slab has 64 blocks);
  *   VEFD_SLAB_PDL=1      programmatic launch between a slab's consecutive kernels
  *                        inside the step graph (measured slower; off). */
 /* The configuration in effect: lattice_tile -1 and post_mode -1 mean the

@@ -83,7 +83,7 @@ struct vefd_ctx {
     // neighbouring slabs; `slab_chunk` steps per replayed graph
     int slabs = -1;  // -1 automatic (slab_count), 0 off
     int slab_chunk = 256;
-    int slab_zs = 12;                      // z-segment of the slab passes (planes marched per block)
+    int slab_zs = 0;                       // z-segment of the slab passes (planes marched per block; 0: slab_segment)
     bool slab_pdl = false;                 // programmatic launch between a slab's consecutive kernels
     cudaStream_t cap = nullptr;            // capture origin
     std::vector<cudaStream_t> slab_s;      // one capture stream per slab
@@ -216,7 +216,7 @@ void carve(vefd_ctx* c) {
     if (const char* e = getenv("VEFD_SCHEDULE")) c->sched = atoi(e) & 3;
     if (const char* e = getenv("VEFD_ZM_SEGMENT")) c->zm_seg_fixed = atoi(e) > 0 ? atoi(e) : 0;
     if (getenv("VEFD_NO_PDL")) c->pdl = false;
-    if (const char* e = getenv("VEFD_SLAB_SEGMENT")) c->slab_zs = atoi(e) > 0 ? atoi(e) : 12;
+    if (const char* e = getenv("VEFD_SLAB_SEGMENT")) c->slab_zs = atoi(e) > 0 ? atoi(e) : 0;
     if (const char* e = getenv("VEFD_SLAB_PDL")) c->slab_pdl = atoi(e) != 0;
 }
 
@@ -421,6 +421,17 @@ int slab_count(const vefd_ctx* c) {
     if (c->slabs >= 0) return c->slabs;
     const int K = c->cfg.ny % 64 == 0 ? 8 : (c->cfg.ny % 32 == 0 ? 4 : 0);
     return slabs_fit(c, K) && c->N / K >= kSlabMinNodes ? K : 1;
+}
+
+// z-segment of the pass on one of K slabs: as long as the slab still gives 64
+// blocks, from 12 to 64 planes.  A segment reads two planes beyond its own, so
+// long ones move fewer bytes; too few blocks leave the SMs waiting for a slab.
+// Steps in us with 12 / 16 / 32 / 64 planes: 128 x 64 x 128 (4 columns a slab) 106 /
+// 113 / 139 / 207, 192 x 64 x 192 (6) 240 / 236 / 244 / 299, 128^3 (8) 208 / 205 / 218 /
+// 276, 256 x 128 x 256 (16) 845 / 837 / 823 / 811, FP16 714 / 705 / 694 / 682.
+int slab_segment(const vefd_ctx* c, int K) {
+    const int columns = c->cfg.nx / 32 * (c->cfg.ny / K / 8), segments = (64 + columns - 1) / columns;
+    return std::max(12, std::min(64, (c->cfg.nz + segments - 1) / segments));
 }
 
 // Everything a captured step bakes into its launches: parameters, kernel
@@ -825,7 +836,7 @@ static vefd_status slab_capture(vefd_ctx* c, int64_t chunk, cudaGraphExec_t* out
     // launch the next one may start its prologue while the previous drains
     // (the cross-slab edges stay full dependencies)
     p0.pdl = c->pdl && c->slab_pdl ? 1 : 0;
-    p0.post_zs = c->slab_zs;
+    p0.post_zs = c->slab_zs > 0 ? c->slab_zs : slab_segment(c, K);
     for (int64_t t = 0; t < chunk && ce == cudaSuccess; ++t) {
         const int par = (int)(t & 1);
         const int cur = c->cur ^ par, ccur = c->ccur ^ (c->fd_on ? par : 0);
