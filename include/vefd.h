@@ -227,7 +227,9 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * lattice_tile selects the node tile the collide-stream kernel (Sec. 2.1,
  * Eqs. 1-3) stages through shared memory: D3Q19 0 = 32x4x2 (default),
  * 1 = 32x2x4, 2 = 32x8x1 nodes (x by y by z); D2Q9 0 = 32x8 (default),
- * 1 = 32x4, 2 = 32x16.  3, 4 and 5 are the same tiles walked by a persistent
+ * 1 = 32x4, 2 = 32x16.  (With tile 0, lattices that fill its tiles badly,
+ * small D2Q9 ones and some of the FP32 moment-space collision take runs of 128
+ * consecutive nodes instead.)  3, 4 and 5 are the same tiles walked by a persistent
  * grid (one block per resident slot on every SM) that double-buffers the
  * staged populations.  post_mode selects how the densities of the new
  * populations and the FENE-P update are done: 0 = a column-marching lattice
@@ -235,9 +237,10 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * followed by a z-marching FENE-P pass that adds the populations which
  * crossed a column side or segment end (D3Q19 with NX % 32 == 0 and
  * NY % 8 == 0; lattice_tile is then unused; it moves fewer bytes but issues
- * about 2.7 times the lattice kernel's instructions); 1 = a 3-D tiled
- * densities/FENE-P pass; 2 (default) = the z-marching densities/FENE-P pass
- * after the tiled lattice kernel; 3 = the tiled lattice kernel (D3Q19 tiles 0
+ * about 2.7 times the lattice kernel's instructions); 1 = a densities/FENE-P
+ * pass over runs of 128 consecutive nodes; 2 (default) = the z-marching
+ * densities/FENE-P pass after the tiled lattice kernel (eager steps of up to
+ * 2^20 nodes take the runs, which are faster there); 3 = the tiled lattice kernel (D3Q19 tiles 0
  * and 1, lattices of whole tiles) also sums, after its collision, the new
  * populations that stay inside its tile into partial densities and writes
  * what it pushes across each face and edge of the tile as per-node partial
@@ -245,7 +248,9 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * (about 3 values per node) instead of reading the new populations back; the
  * partial sums use the staging planes, which are free inside a step.  Post
  * modes 1 and 2 with tiles 0-2 run the same arithmetic in the
- * same order and give bit-identical results; the persistent tiles (separately
+ * same order and give bit-identical results (with the FP32 moment-space
+ * collision on lattices the column does not fit, tile 0 agrees with tiles 1
+ * and 2 to FP32 rounding); the persistent tiles (separately
  * compiled, multiply-adds contracted as the compiler sees fit) and post modes 0
  * and 3 (each node's new density summed in another order) agree to FP32
  * rounding.  A tile the lattice shape
@@ -259,7 +264,7 @@ vefd_status vefd_set_kernel_config(vefd_ctx *ctx, int lattice_tile, int post_mod
  * and testing; the defaults are the measured fastest, and results stay
  * within the agreements stated above):
  *   VEFD_NO_TMA=1        unstaged kernels only;
- *   VEFD_NO_ZMARCH=1     the 3-D tiled densities pass instead of the z-marching one;
+ *   VEFD_NO_ZMARCH=1     the densities pass over runs of nodes instead of the z-marching one;
  *   VEFD_NO_FUSED=1      post_mode 0 runs as post_mode 2;
  *   VEFD_NO_PDL=1        no programmatic dependent launch between a step's kernels;
  *   VEFD_SCHEDULE=b      bit 0 walks the lattice kernel's tiles, bit 1 the pass's
@@ -296,14 +301,16 @@ vefd_status vefd_autotune(vefd_ctx *ctx, int steps, double *times_ms);
  *   of step n on slabs k-1, k, k+1, and its pass of step n waits for the
  *   lattice kernels of step n on those slabs.  Work on different slabs then
  *   overlaps, and a slab's new populations can be re-read while still in L2.
- *   Each slab's pass marches z-segments of 12 planes (shorter blocks than
- *   the whole-lattice pass, so the pass its neighbours wait for finishes
- *   sooner).  This form needs: D3Q19; a staged tile 0-2 with post mode 2;
+ *   Each slab's pass marches z-segments of 12 to 64 planes, as long as they
+ *   leave the slab 64 blocks.  This form needs: D3Q19; a staged tile 0-2 with post mode 2;
  *   NY a multiple of 8 * slabs.  An explicit slab count the lattice does not
  *   admit means eager stepping.
  * - Whole-lattice (slabs = 1): the eager launch pairs of `chunk` steps,
  *   replayed as one graph; any lattice and kernel choice.  It saves the
- *   host-side launch cost, which bounds small lattices.
+ *   host-side launch cost, which bounds small lattices.  With the automatic
+ *   setting and kernel choice, D2Q9 lattices of up to 8192 nodes take calls of
+ *   four steps and more in launches of up to 1024 steps instead, which hold
+ *   the state in shared memory and leave the same bits.
  * In both forms the kernels and their per-node arithmetic are those of the
  * eager step, so results are bit-identical.  slabs = 0 turns the graph off;
  * slabs = -1 (the default) chooses 8 slabs when NY is a multiple of 64, 4 when

@@ -9,8 +9,9 @@
 //                 the densities/FD pass, velocity (Eq. equilibrium:vel),
 //                 viscosity (Eq. smoothingvisco), forced collision (Eq. LB)
 //                 and push streaming with half-way bounce-back on moving walls.
-//                 Populations held in registers; used for any lattice size and
-//                 for the macroscopic (non-streaming) passes.
+//                 Runs of 128 consecutive nodes with the populations in registers;
+//                 for lattices that fill boxes badly, small ones, and the
+//                 macroscopic (non-streaming) passes.
 //   k_lattice_tma the same step for lattices whose rows are 16-byte multiples:
 //                 one TMA copy stages the block's populations (all components
 //                 and directions of a 32 x BY x BZ tile) in shared memory while
@@ -20,7 +21,7 @@
 //   k_lattice_pers persistent form of k_lattice_tma with two staging buffers.
 // The collision (template COLL) is the single-relaxation-time form of
 // Eq. (LB) (0) or its moment-space form with the paper's relaxation times (1).
-// One thread per node; a warp covers 32 consecutive x, so every population
+// One thread per node; a warp covers 32 consecutive nodes, so every population
 // plane is read and written as contiguous 128-byte rows (writes of moving
 // populations are shifted by one element in x).
 #include <cuda.h>

@@ -24,13 +24,17 @@
 // Sums over K run tap by tap, 16 channels at a time, in the order of the
 // im2col product (the prediction's bits are those of that product).
 //
-// Measured, 64^3 unless said: the prediction 368 us (explicit im2col matrices and
-// their scalar kernels: 12263); 48 -> 16 channels forward and backward 175 us
-// (6742), of it 43 us forward, 62 us weight gradient, 32 us data gradient, 37 us
-// conversion, mask and sums; 232 -> 80 at 16^3 115 us (780), 49 us forward: one
-// chain of 392 steps a tile at about 85 clocks a step, which bounds the deep
-// levels; the fine ones are bound by the tensor core's 39 clocks a step of 16
-// columns (22 us of the 43) and the staging of 16-byte pieces.
+// Measured, 64^3 unless said: the prediction 330 us (explicit im2col matrices and
+// their scalar kernels: 12263); 48 -> 16 channels forward and backward 171 us
+// (6742), of it 43 us forward, 61 us weight gradient, 31 us data gradient, 36 us
+// conversion, mask and sums; 232 -> 80 at 16^3 101 us (780).  Deep levels are one
+// chain a tile: at 16^3 392 steps on one accumulator at 85 clocks, beside which
+// setup (2k clocks), the halo's 9000 pieces (10k), and 49 chunks of weights count;
+// the fine levels are bound by the tensor core's 39 clocks a step of 16 columns
+// (22 us of the 43) and the staging of 16-byte pieces.  What made the chain
+// shorter: weights of part of the columns by one box a chunk instead of 2 x chunk
+// small copies (forward at 16^3 49.0 to 42.2 us together with halo planes that
+// land in three groups), and waits of one poll (prediction 345 to 330 us).
 #include <algorithm>
 #include <cmath>
 
@@ -980,7 +984,7 @@ cudaError_t launch_conv(int kind, const void* A, int B, int D, int H, int W, int
     CUtensorMap tm0, tm1, tmw{};
     if (!halo_maps(&tm0, &tm1, A, h, p.groups == 1 ? h.hz : 1)) return cudaErrorInvalidValue;
     if (p.bn < Np && !weight_map(&tmw, wk, (long long)h.nblk * e.npairs * 2, Np, p.bn, p.chunk * 2)) return cudaErrorInvalidValue;
-    static const cudaError_t err = cudaFuncSetAttribute(k_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    const cudaError_t err = cudaFuncSetAttribute(k_conv, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (err != cudaSuccess) return err;
     const int vec = N % 4 == 0 && (reinterpret_cast<uintptr_t>(Y) & 15u) == 0;
     k_conv<<<grid, kConvThreads, p.smem, st>>>(tm0, tm1, tmw, h, e, (const uint4*)wk, Np, p.bn, p.nbuf, p.nset,

@@ -370,9 +370,10 @@ uint64_t splitmix64(uint64_t seed, uint64_t i) {
 //   27.5 us both, 132 x 70 x 100 (0.80) 63.0 against 67.7, 68 x 36 x 50 (0.71)
 //   14.4 against 13.6.
 // - D3Q19, moment-space collision: 16-bit storage always (256 x 128 x 64 108
-//   against 112 us, 116 x 50 x 70 26.7 and 27.1), FP32 never (64^3 20.7 us in
-//   boxes, 19.7 in runs; 128 x 64 x 128 68.4 and 65.7, 132 x 70 x 100 73.2 and
-//   59.8).
+//   against 112 us, 116 x 50 x 70 26.7 and 27.1), FP32 where the z-marching column
+//   fits: runs are faster (64^3 20.7 us in boxes, 19.7 in runs; 132 x 70 x 100 73.2
+//   and 59.8) but may round the moving-wall term differently, and lattices that
+//   the slab graph and the ensembles take give the same bits on every route.
 bool lattice_boxes(const vefd_ctx* c) {
     if (!c->tma_ok) return false;
     if (c->lat_tile != 0 || c->parts_ok) return true;
@@ -382,7 +383,7 @@ bool lattice_boxes(const vefd_ctx* c) {
                             ((c->cfg.nz + bz - 1) / bz);
     const double fill = (double)c->N / ((double)boxes * bx * by * bz);
     if (c->D == 2) return c->N >= (1 << 18) && fill >= 0.75;
-    if (c->collision == 1) return c->cfg.precision != 0;
+    if (c->collision == 1) return c->cfg.precision != 0 || post_zm_eligible(c->cfg.lattice, c->cfg.nx, c->cfg.ny);
     return fill >= 0.75;
 }
 
@@ -461,9 +462,9 @@ bool slab_usable(vefd_ctx* c) {
 
 // Whether several steps run in one launch (launch_small): a D2Q9 lattice of as
 // many nodes as its cluster has threads, with the automatic step graph and
-// kernel choice.  The launch is the faster form up to that size (lbm_small.cu).
-bool small_usable(const vefd_ctx* c) {
-    return c->D == 2 && c->N <= kSmallMaxNodes && c->slabs < 0 && c->lat_tile == 0 && !c->prof_on;
+// kernel choice, on a stream that is not being captured.  The launch is the faster form up to that size (lbm_small.cu).
+bool small_usable(vefd_ctx* c) {
+    return c->D == 2 && c->N <= kSmallMaxNodes && c->slabs < 0 && c->lat_tile == 0 && slab_usable(c);
 }
 
 // Records an event pair around one launch when kernel timing is on.

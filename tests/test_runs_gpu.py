@@ -1,5 +1,5 @@
 """The step over runs of consecutive nodes (the form of tile 0 where boxes fill
-badly, of small D2Q9 lattices and of the FP32 moment-space collision) gives the
+badly, of small D2Q9 lattices and of the FP32 moment-space collision off the column) gives the
 bits of the staged boxes (to rounding in the moment-space collision), also where the last run is partial, a run spans
 several planes, or the whole lattice is less than one run."""
 import numpy as np
