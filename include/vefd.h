@@ -240,7 +240,7 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * about 2.7 times the lattice kernel's instructions); 1 = a densities/FENE-P
  * pass over runs of 128 consecutive nodes; 2 (default) = the z-marching
  * densities/FENE-P pass after the tiled lattice kernel (eager steps of up to
- * 2^20 nodes take the runs, which are faster there); 3 = the tiled lattice kernel (D3Q19 tiles 0
+ * 786432 nodes take the runs, which are faster there); 3 = the tiled lattice kernel (D3Q19 tiles 0
  * and 1, lattices of whole tiles) also sums, after its collision, the new
  * populations that stay inside its tile into partial densities and writes
  * what it pushes across each face and edge of the tile as per-node partial

@@ -392,10 +392,11 @@ bool lattice_boxes(const vefd_ctx* c) {
 // 7, which pays once the pass is bound by memory; below, its segments are short
 // and its blocks few.  Steps in us, runs / columns: 32^3 6.5 / 9.0, 64 x 32 x 32
 // 9.2 / 11.8, 64^3 25.5 / 26.1 (FP16 22.6 / 24.8), 128 x 64 x 64 56.6 / 58.7,
+// 128 x 64 x 96 85.9 / 85.3 (FP16 72.3 / 72.8),
 // 128 x 64 x 128 112.9 / 113.5 (FP16 95.2 / 96.4), 160 x 72 x 128 160.6 / 160.3,
 // 224 x 104 x 128 316 / 303 (FP16 269 / 263).  (The slab graph and the
 // batched ensembles march columns at every size.)
-constexpr long long kRunsMaxNodes = 1 << 20;
+constexpr long long kRunsMaxNodes = 3 << 18;
 bool post_columns(const vefd_ctx* c) { return c->zm_ok && (c->parts_ok || c->N > kRunsMaxNodes); }
 
 // The pipelined y-slab split applies for K slabs: staged lattice tiles (not
