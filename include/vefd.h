@@ -239,8 +239,9 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * NY % 8 == 0; lattice_tile is then unused; it moves fewer bytes but issues
  * about 2.7 times the lattice kernel's instructions); 1 = a densities/FENE-P
  * pass over runs of 128 consecutive nodes; 2 (default) = the z-marching
- * densities/FENE-P pass after the tiled lattice kernel (eager steps of up to
- * 786432 nodes take the runs, which are faster there); 3 = the tiled lattice kernel (D3Q19 tiles 0
+ * densities/FENE-P pass after the tiled lattice kernel (while this function
+ * has not been called, eager steps of up to 786432 nodes take the runs of mode
+ * 1 instead, which are faster there; set, mode 2 marches at every size); 3 = the tiled lattice kernel (D3Q19 tiles 0
  * and 1, lattices of whole tiles) also sums, after its collision, the new
  * populations that stay inside its tile into partial densities and writes
  * what it pushes across each face and edge of the tile as per-node partial
@@ -275,11 +276,15 @@ vefd_status vefd_set_kernel_config(vefd_ctx *ctx, int lattice_tile, int post_mod
  *   VEFD_SLAB_PDL=1      programmatic launch between a slab's consecutive kernels
  *                        inside the step graph (measured slower; off). */
 /* The configuration in effect: lattice_tile -1 and post_mode -1 mean the
- * unstaged kernels; post_mode 1 also when the column does not fit. */
+ * unstaged kernels; post_mode 1 also when the column does not fit, 2 also for
+ * the default where its eager steps take the runs. */
 vefd_status vefd_get_kernel_config(const vefd_ctx *ctx, int *lattice_tile, int *post_mode);
 /* Times every admitted (lattice_tile, post_mode) pair for `steps` steps on a
- * scratch lattice of the same configuration and parameters (droplet initial
- * state; the context's own state is untouched), then applies the fastest.
+ * scratch lattice of the same configuration, parameters and step-graph setting
+ * (droplet initial state; the context's own state is untouched), then applies
+ * the fastest.  The steps are one vefd_step call after an untimed one, so a
+ * pair is timed with the step graph or the many-step launches that it admits
+ * (D2Q9 lattices of up to 8192 nodes: four steps at least).
  * times_ms (host, 18 doubles or NULL) receives the times, index
  * post_mode * 6 + lattice_tile, -1 for pairs not admitted (post_mode 0 is
  * timed with lattice_tile 0 only; post_mode 3 is not timed: its lattice
@@ -308,7 +313,7 @@ vefd_status vefd_autotune(vefd_ctx *ctx, int steps, double *times_ms);
  * - Whole-lattice (slabs = 1): the eager launch pairs of `chunk` steps,
  *   replayed as one graph; any lattice and kernel choice.  It saves the
  *   host-side launch cost, which bounds small lattices.  With the automatic
- *   setting and kernel choice, D2Q9 lattices of up to 8192 nodes take calls of
+ *   setting and lattice_tile 0, D2Q9 lattices of up to 8192 nodes take calls of
  *   four steps and more in launches of up to 1024 steps instead, which hold
  *   the state in shared memory and leave the same bits.
  * In both forms the kernels and their per-node arithmetic are those of the

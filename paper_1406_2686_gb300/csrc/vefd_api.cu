@@ -62,6 +62,7 @@ struct vefd_ctx {
     bool tma_ok = false;
     int lat_tile = 0;                      // staged tile shape of the lattice kernel (lattice_tile_shape)
     int post_mode = 2;                     // 0 column march with fused densities, 1 runs of nodes, 2 separate z-march pass
+    bool post_auto = true;                 // no post mode was set: mode 2, eager steps in runs where they are faster (post_columns)
     // tensor maps with a 32 x 8 x 1 box for the z-marching densities/FD pass
     alignas(64) CUtensorMap tmap_zm[2];
     bool zm_ok = false;
@@ -387,17 +388,19 @@ bool lattice_boxes(const vefd_ctx* c) {
     return fill >= 0.75;
 }
 
-// Whether the densities/FENE-P pass marches columns along z (else runs of 128
-// consecutive nodes).  The march reads every stencil value 1.3 times instead of
+// Whether the densities/FENE-P pass of an eager step marches columns along z
+// (else runs of 128 consecutive nodes): as post mode 2 says where it was set, by
+// size where nothing was.  The march reads every stencil value 1.3 times instead of
 // 7, which pays once the pass is bound by memory; below, its segments are short
 // and its blocks few.  Steps in us, runs / columns: 32^3 6.5 / 9.0, 64 x 32 x 32
 // 9.2 / 11.8, 64^3 25.5 / 26.1 (FP16 22.6 / 24.8), 128 x 64 x 64 56.6 / 58.7,
 // 128 x 64 x 96 85.9 / 85.3 (FP16 72.3 / 72.8),
 // 128 x 64 x 128 112.9 / 113.5 (FP16 95.2 / 96.4), 160 x 72 x 128 160.6 / 160.3,
-// 224 x 104 x 128 316 / 303 (FP16 269 / 263).  (The slab graph and the
-// batched ensembles march columns at every size.)
+// 224 x 104 x 128 316 / 303 (FP16 269 / 263).  From 786432 to 1048576 nodes the two
+// are within 1.3 % of each other, in either direction; the line lies at the lower
+// end.  (The slab graph and the batched ensembles march columns at every size.)
 constexpr long long kRunsMaxNodes = 3 << 18;
-bool post_columns(const vefd_ctx* c) { return c->zm_ok && (c->parts_ok || c->N > kRunsMaxNodes); }
+bool post_columns(const vefd_ctx* c) { return c->zm_ok && (c->parts_ok || !c->post_auto || c->N > kRunsMaxNodes); }
 
 // The pipelined y-slab split applies for K slabs: staged lattice tiles (not
 // the persistent forms) with the separate z-marching pass, D3Q19, and rows
@@ -442,7 +445,7 @@ std::vector<double> state_key(const vefd_ctx* m) {
     return {m->u_wall, m->fext[0], m->fext[1], m->fext[2], m->tau_p, m->eta_p, m->L2, m->kappa,
             (double)m->phase, (double)m->fd_on, (double)m->coupling, (double)m->collision, (double)m->chol,
             m->rho_ref[0], m->rho_ref[1], (double)m->lat_tile, (double)m->tma_ok, (double)m->zm_ok,
-            (double)m->fused_ok, (double)m->parts_ok, (double)(m->drho < m->drho_alt), (double)m->sched,
+            (double)m->fused_ok, (double)m->parts_ok, (double)m->post_auto, (double)(m->drho < m->drho_alt), (double)m->sched,
             (double)m->cur,
             (double)m->ccur, (double)m->have_prev, (double)m->drho_valid, (double)m->pdl,
             (double)(uintptr_t)m->mem, (double)m->zm_seg_fixed, (double)slab_count(m), (double)m->slab_chunk};
@@ -463,10 +466,9 @@ bool slab_usable(vefd_ctx* c) {
 
 // Whether several steps run in one launch (launch_small): a D2Q9 lattice of as
 // many nodes as its cluster has threads, with the automatic step graph and
-// kernel choice, on a stream that is not being captured.  The launch is the faster form up to that size (lbm_small.cu).
-bool small_usable(vefd_ctx* c) {
-    return c->D == 2 && c->N <= kSmallMaxNodes && c->slabs < 0 && c->lat_tile == 0 && slab_usable(c);
-}
+// tile 0, on a stream that is not being captured.  The launch is the faster form up to that size (lbm_small.cu).
+bool small_nodes(const vefd_ctx* c) { return c->D == 2 && c->N <= kSmallMaxNodes; }
+bool small_usable(vefd_ctx* c) { return small_nodes(c) && c->slabs < 0 && c->lat_tile == 0 && slab_usable(c); }
 
 // Records an event pair around one launch when kernel timing is on.
 struct ProfScope {
@@ -1429,6 +1431,7 @@ vefd_status vefd_set_kernel_config(vefd_ctx* c, int lattice_tile, int post_mode)
     if (post_mode < 0 || post_mode > 3) return fail(c, VEFD_ERR_ARG, "post_mode must be 0, 1, 2 or 3");
     c->lat_tile = lattice_tile;
     c->post_mode = post_mode;
+    c->post_auto = false;
     if (c->mem) build_tensor_maps(c);
     return VEFD_OK;
 }
@@ -1453,7 +1456,11 @@ vefd_status vefd_autotune(vefd_ctx* c, int steps, double* times_ms) {
     vefd_ctx* t = nullptr;
     vefd_status st = vefd_create(&cfg, c->stream, &t);
     if (st != VEFD_OK) return fail(c, st, "autotune: cannot create the scratch lattice");
-    t->slabs = 0;  // the kernels are timed one launch pair at a time
+    // timed as vefd_step of the context runs them: a choice may admit the slab
+    // graph or the many-step launches, or lose them
+    t->slabs = c->slabs;
+    t->slab_chunk = c->slab_chunk;
+    const int timed = small_nodes(c) ? std::max(steps, (int)kSmallMinSteps) : steps;
     t->u_wall = c->u_wall;
     for (int k = 0; k < 3; ++k) t->fext[k] = c->fext[k];
     t->tau_p = c->tau_p;
@@ -1475,7 +1482,7 @@ vefd_status vefd_autotune(vefd_ctx* c, int steps, double* times_ms) {
     }
     if (st == VEFD_OK) st = vefd_step(t, 2);
     double best = 1e300;
-    int best_tile = c->lat_tile, best_post = c->post_mode;
+    int best_tile = 0, best_post = -1;  // -1: no pair admitted, nothing to apply
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (st == VEFD_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = VEFD_ERR_CUDA;
     for (int pm = 0; pm < 3 && st == VEFD_OK; ++pm)
@@ -1485,10 +1492,10 @@ vefd_status vefd_autotune(vefd_ctx* c, int steps, double* times_ms) {
             vefd_set_kernel_config(t, tile, pm);
             if (!t->tma_ok) continue;
             if (pm == 0 && (!t->fused_ok || tile != 0)) continue;  // the column march has its own tile
-            st = vefd_step(t, 2);  // warm the configuration
+            st = vefd_step(t, timed);  // untimed: captures the graphs that the timed call replays
             if (st != VEFD_OK) break;
             cudaEventRecord(e0, t->stream);
-            st = vefd_step(t, steps);
+            st = vefd_step(t, timed);
             cudaEventRecord(e1, t->stream);
             if (st != VEFD_OK || cudaEventSynchronize(e1) != cudaSuccess) {
                 st = st != VEFD_OK ? st : VEFD_ERR_CUDA;
@@ -1513,7 +1520,7 @@ vefd_status vefd_autotune(vefd_ctx* c, int steps, double* times_ms) {
         return fail(c, st, "autotune failed: %s", why.c_str());
     }
     vefd_destroy(t);
-    return vefd_set_kernel_config(c, best_tile, best_post);
+    return best_post < 0 ? VEFD_OK : vefd_set_kernel_config(c, best_tile, best_post);
 }
 
 // ---- ensembles --------------------------------------------------------------
