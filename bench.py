@@ -544,7 +544,6 @@ def time_ensemble(steps, warmup, chunk=32, setups=None, label=None):
         lats = build()
         E = vefd.Ensemble(lats, stream)
         E.set_batched(batched)
-        E.set_groups(4 if batched else 0)  # the automatic count; setting it keeps the batched form
         E.step(warmup, chunk)
         E.step(chunk, chunk)  # captures the ensemble's chunk graph before the timed region
         torch.cuda.synchronize()

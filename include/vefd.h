@@ -380,9 +380,10 @@ vefd_status vefd_ensemble_create(vefd_ctx *const *members, int n, void *stream, 
  * member is not initialised, VEFD_ERR_CUDA on capture or launch errors
  * (see vefd_ensemble_last_error). */
 vefd_status vefd_ensemble_step(vefd_ensemble *ens, int64_t nsteps, int64_t chunk);
-/* Batched launches (default on; used for members of fewer than 2^14 or more
- * than 2^19 nodes on average, or once a z-segment, group count or lattice tile
- * is set): when every member is D3Q19 with the same
+/* Batched launches.  Until this function or vefd_ensemble_set_config is called
+ * (the automatic form, reported as on), members of fewer than 2^14 or more than
+ * 2^19 nodes on average take them, and others once a z-segment, a group count
+ * or lattice tile 1 is set.  on = 1 takes them at every size: when every member is D3Q19 with the same
  * component count, storage type, collision operator, FENE-P switch and
  * programmatic-launch setting, and each takes the staged lattice kernel and
  * the separate z-marching densities/FENE-P pass (NX % 32 == 0, NY % 8 == 0,
@@ -405,7 +406,7 @@ vefd_status vefd_ensemble_set_batched(vefd_ensemble *ens, int on);
 /* 1 when the currently captured graph uses the batched launches, else 0. */
 int vefd_ensemble_is_batched(const vefd_ensemble *ens);
 /* Kernel choices of the replayed steps: batched (0/1, as
- * vefd_ensemble_set_batched) and the z-segment length, in planes, of the
+ * vefd_ensemble_set_batched; reported as 1 for the automatic form) and the z-segment length, in planes, of the
  * batched densities/FENE-P pass (0: automatic, the length that fills two
  * blocks per SM with the fewest planes per block; otherwise clamped to each
  * member's NZ).  Results do not depend on the segment length.  Takes effect
@@ -415,7 +416,7 @@ vefd_status vefd_ensemble_set_config(vefd_ensemble *ens, int batched, int post_s
 vefd_status vefd_ensemble_get_config(const vefd_ensemble *ens, int *batched, int *post_segment);
 /* Group count of the batched launches (no counterpart in the paper; a
  * launch-layout choice): 0 (the default) means 4; otherwise 1..64, clamped to
- * the member count.  Members are split into that many contiguous groups of
+ * the member count, and the automatic form is the batched one.  Members are split into that many contiguous groups of
  * about equal node count, each group one graph branch of two launches per
  * step.  Results do not depend on the group count (bit-identical).  Takes
  * effect at the next replay (after waiting for earlier replays).
@@ -424,7 +425,8 @@ vefd_status vefd_ensemble_set_groups(vefd_ensemble *ens, int groups);
 /* The group-count setting (0: automatic). */
 vefd_status vefd_ensemble_get_groups(const vefd_ensemble *ens, int *groups);
 /* Lattice tiles of the batched launches (no counterpart in the paper; a launch
- * shape): 0 (default) 32 x 4 x 2 nodes, 1 32 x 8 x 1.  Results agree with
+ * shape): 0 (default) 32 x 4 x 2 nodes, 1 32 x 8 x 1, with which the
+ * automatic form is the batched one.  Results agree with
  * vefd_step to FP32 rounding for both.  Takes effect at the next replay (after
  * waiting for earlier replays).  VEFD_ERR_ARG for a NULL ensemble or another
  * value. */
@@ -434,7 +436,7 @@ vefd_status vefd_ensemble_get_tile(const vefd_ensemble *ens, int *tile);
  * branches; and batched launches with each lattice tile (0, 1), each with the
  * automatic z-segment of the densities pass, twice it and half of it.
  * Each is timed as `steps` replayed steps (after one untimed replay that
- * captures it), and the fastest is kept.  The timed steps are real steps:
+ * captures it), and the fastest is kept (set as by vefd_ensemble_set_config).  The timed steps are real steps:
  * every member advances by 7 (steps + chunk) steps (plus one eager step if its
  * Euler start is pending), its results those of vefd_step to FP32 rounding.
  * times_ms (7 slots, or NULL) receives each configuration's milliseconds, -1

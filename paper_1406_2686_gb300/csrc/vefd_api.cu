@@ -1527,6 +1527,10 @@ vefd_status vefd_autotune(vefd_ctx* c, int steps, double* times_ms) {
 
 }  // extern "C"
 
+// Form of an ensemble's replayed steps: by the members' size until the caller
+// sets one; batched launches only where the members allow them.
+enum class EnsForm { automatic, branches, batched };
+
 struct vefd_ensemble {
     std::vector<vefd_ctx*> members;
     std::vector<cudaStream_t> branch;  // one capture/eager branch per member
@@ -1541,7 +1545,7 @@ struct vefd_ensemble {
     std::string err;
     // batched launches: one lattice kernel and one densities/FENE-P pass per
     // step over the tiles of all members, from a device table of members
-    int batched_pref = 1;       // use them when the members allow
+    EnsForm form = EnsForm::automatic;
     int post_seg = 0;           // z-segment of the batched densities pass: 0 automatic, else planes
     int tile = 0;               // batched lattice tiles: 0 32 x 4 x 2, 1 32 x 8 x 1
     bool batched = false;       // the captured graph uses them
@@ -1834,15 +1838,17 @@ void ens_sets(const vefd_ensemble* e, std::vector<int>* order, std::vector<int>*
     first->push_back(n);
 }
 
-// Whether the branch form is taken although the members admit batched
-// launches: their mean size is 2^14 to 2^19 nodes and nothing was set.  Smaller
+// Whether the automatic form is that of branches although the members admit
+// batched launches: their mean size is 2^14 to 2^19 nodes and no z-segment, group
+// count or tile 1 was set.  Smaller
 // ones are bound by their launches (64 of 32 x 16 x 16: 61 us batched, 49 in sets, but
 // four times the graph), larger ones gain nothing (2 of 128 x 64 x 128 217 / 219).
 bool ens_prefers_sets(const vefd_ensemble* e) {
     long long total = 0;
     for (const vefd_ctx* m : e->members) total += m->N;
     const long long n = (long long)e->members.size();
-    return n >= 2 && e->post_seg == 0 && e->groups == 0 && e->tile == 0 && total >= n << 14 && total <= n << 19;
+    return e->form == EnsForm::automatic && n >= 2 && e->post_seg == 0 && e->groups == 0 && e->tile == 0 &&
+           total >= n << 14 && total <= n << 19;
 }
 
 // Steps of one captured graph of the branch form: the largest even divisor of
@@ -2010,7 +2016,7 @@ vefd_status vefd_ensemble_step(vefd_ensemble* e, int64_t nsteps, int64_t chunk) 
         if (stale) {
             if (e->exec) cudaGraphExecDestroy(e->exec);
             e->exec = nullptr;
-            const bool batched = e->batched_pref && ens_batchable(e) && !ens_prefers_sets(e);
+            const bool batched = e->form != EnsForm::branches && ens_batchable(e) && !ens_prefers_sets(e);
             e->span = batched ? chunk : ens_span(chunk);
             const vefd_status st = batched ? ens_capture_batched(e, chunk) : ens_capture(e, e->span);
             if (st != VEFD_OK) return st;
@@ -2029,24 +2035,28 @@ vefd_status vefd_ensemble_step(vefd_ensemble* e, int64_t nsteps, int64_t chunk) 
     return ens_eager(e, nsteps - full * chunk);
 }
 
-vefd_status vefd_ensemble_set_config(vefd_ensemble* e, int batched, int post_segment) {
-    if (!e || (batched != 0 && batched != 1) || post_segment < 0) return VEFD_ERR_ARG;
-    if (e->batched_pref != batched || e->post_seg != post_segment) {
+static void ens_set_form(vefd_ensemble* e, EnsForm form, int post_segment) {
+    if (e->form != form || e->post_seg != post_segment) {
         // the next replay re-captures; earlier replays may still be in flight
         if (e->exec) {
             cudaStreamSynchronize(e->main);
             cudaGraphExecDestroy(e->exec);
         }
         e->exec = nullptr;
-        e->batched_pref = batched;
+        e->form = form;
         e->post_seg = post_segment;
     }
+}
+
+vefd_status vefd_ensemble_set_config(vefd_ensemble* e, int batched, int post_segment) {
+    if (!e || (batched != 0 && batched != 1) || post_segment < 0) return VEFD_ERR_ARG;
+    ens_set_form(e, batched ? EnsForm::batched : EnsForm::branches, post_segment);
     return VEFD_OK;
 }
 
 vefd_status vefd_ensemble_get_config(const vefd_ensemble* e, int* batched, int* post_segment) {
     if (!e || !batched || !post_segment) return VEFD_ERR_ARG;
-    *batched = e->batched_pref;
+    *batched = e->form != EnsForm::branches;
     *post_segment = e->post_seg;
     return VEFD_OK;
 }
@@ -2123,7 +2133,8 @@ vefd_status vefd_ensemble_autotune(vefd_ensemble* e, int64_t steps, int64_t chun
         if (e0) cudaEventDestroy(e0);
         return ens_fail(e, VEFD_ERR_CUDA, "cannot create timing events");
     }
-    const int keep_b = e->batched_pref, keep_s = e->post_seg, keep_t = e->tile;
+    const EnsForm keep_f = e->form;
+    const int keep_s = e->post_seg, keep_t = e->tile;
     vefd_status st = VEFD_OK;
     double best = 1e300;
     int best_k = -1;
@@ -2151,7 +2162,7 @@ vefd_status vefd_ensemble_autotune(vefd_ensemble* e, int64_t steps, int64_t chun
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st != VEFD_OK || best_k < 0) {
-        vefd_ensemble_set_config(e, keep_b, keep_s);
+        ens_set_form(e, keep_f, keep_s);
         vefd_ensemble_set_tile(e, keep_t);
         return st != VEFD_OK ? st : ens_fail(e, VEFD_ERR_CUDA, "no configuration was timed");
     }

@@ -588,8 +588,8 @@ class Ensemble:
         vefd_ensemble_step(self.ens, n, chunk)
 
     def set_batched(self, on):
-        """One launch per kernel phase over all members where that is the
-        faster form (default), or always one graph branch per member."""
+        """One launch per kernel phase over all members where they allow it, or
+        one graph branch per member; until set, by the members' size."""
         vefd_ensemble_set_batched(self.ens, 1 if on else 0)
 
     @property

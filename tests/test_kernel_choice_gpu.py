@@ -78,3 +78,27 @@ def test_autotune_times_the_step_graph():
     names = launched(lambda: L.autotune(steps=8))
     # eager, each of 6 tiles (and the fused pair) would launch it 16 times: 112
     assert names["k_post_zm"] >= 3 * 16 * 4, names
+
+
+def test_ensemble_form_set_is_the_form_that_runs():
+    """Members of 2^14 nodes and more step in branches until batched launches are
+    set, which then run, also with tile 0 and the automatic segment and groups."""
+    from paper_1406_2686_gb300 import vefd
+    sizes = [(64, 32, 16), (32, 32, 33), (64, 16, 20)]
+    boxes = [dict(COMMON, lattice=1, nx=x, ny=y, nz=z, ncomp=2, walls=1, u_wall=0.03) for x, y, z in sizes]
+    E = vefd.Ensemble([make(b, seed=30 + k) for k, b in enumerate(boxes)])
+    for ask, batched in ((None, False), (True, True), (False, False)):
+        if ask is not None:
+            E.set_batched(ask)
+        E.step(9, chunk=4)
+        assert E.batched == batched and E.config == (0 if ask is False else 1, 0)
+    E.set_config(True, 0)
+    E.step(4, chunk=4)
+    assert E.batched
+    times = E.autotune(steps=8, chunk=4)
+    assert all(t > 0 for t in times), times  # every configuration: the members allow batched launches
+    best = int(np.argmin(times))
+    assert E.config[0] == int(best > 0)
+    E.step(8, chunk=4)
+    assert E.batched == (best > 0)
+    E.close()
