@@ -452,13 +452,9 @@ cudaError_t post_zm(const CUtensorMap* tm, const StepParams& p, const StepBufs& 
                     Parts parts = Parts{}) {
     constexpr bool FUSED = MODE == 1;
     constexpr int smem = MODE != 0 ? 4 * kZmPlane * (int)sizeof(float) : zm_smem_bytes<PT, NCOMP>();
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e =
-            cudaFuncSetAttribute(k_post_zm<PT, NCOMP, FD, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice site;
+    const cudaError_t e = allow_smem(site, k_post_zm<PT, NCOMP, FD, MODE>, smem);
+    if (e != cudaSuccess) return e;
     if (!g_sm_count) {
         int dev = 0;
         cudaGetDevice(&dev);
@@ -520,12 +516,9 @@ template <class PT, int NCOMP, bool FD>
 cudaError_t post_batch(const EnsMember* members, const int* start, int nm, int items, int parity, bool pdl,
                        cudaStream_t s) {
     constexpr int smem = zm_smem_bytes<PT, NCOMP>();
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_post_batch<PT, NCOMP, FD>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice site;
+    const cudaError_t e = allow_smem(site, k_post_batch<PT, NCOMP, FD>, smem);
+    if (e != cudaSuccess) return e;
     return launch_pdl(pdl, k_post_batch<PT, NCOMP, FD>, dim3(items), dim3(kZmBX, kZmBY, 1), smem, s, members, start,
                       nm, parity);
 }

@@ -1217,17 +1217,16 @@ template <class PT, class L, int NCOMP, int BX, int BY, int BZ>
 cudaError_t launch_pers_tile(const CUtensorMap* tm, const StepParams& p, const StepBufs& b, int rev, cudaStream_t s) {
     constexpr int T = BX * BY * BZ;
     constexpr int smem = 2 * NCOMP * (L::Q - 1) * T * (int)sizeof(PT);
-    static int per_sm = 0;  // resident blocks per SM of this instantiation
-    if (!per_sm) {
-        cudaError_t e = cudaFuncSetAttribute(k_lattice_pers<PT, L, NCOMP, BX, BY, BZ>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_lattice_pers<PT, L, NCOMP, BX, BY, BZ>, T, smem);
-        if (e != cudaSuccess) return e;
-        if (nb < 1) return cudaErrorInvalidConfiguration;
-        per_sm = nb;
-    }
+    static PerDevice site;
+    int per_sm = 0;  // resident blocks per SM of this instantiation
+    const cudaError_t e = site.get(&per_sm, [&](int* nb) {
+        cudaError_t err = cudaFuncSetAttribute(k_lattice_pers<PT, L, NCOMP, BX, BY, BZ>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (err != cudaSuccess) return err;
+        err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, k_lattice_pers<PT, L, NCOMP, BX, BY, BZ>, T, smem);
+        return err == cudaSuccess && *nb < 1 ? cudaErrorInvalidConfiguration : err;
+    });
+    if (e != cudaSuccess) return e;
     const int ntx = (p.nx + BX - 1) / BX, nty = (p.ny + BY - 1) / BY, ntz = (p.nz + BZ - 1) / BZ;
     const long long ntiles = (long long)ntx * nty * ntz;
     const long long grid = std::min<long long>(ntiles, (long long)per_sm * lattice_sm_count());
@@ -1249,13 +1248,9 @@ inline int zm_segment_length(const StepParams& p) {
 template <class PT, int NCOMP, int COLL>
 cudaError_t launch_zm(const CUtensorMap* tm, const StepParams& p, const StepBufs& b, int zs, int rev, cudaStream_t s) {
     constexpr int smem = 2 * NCOMP * 18 * 256 * (int)sizeof(PT);  // two staged planes
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_lattice_zm<PT, NCOMP, COLL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice site;
+    const cudaError_t e = allow_smem(site, k_lattice_zm<PT, NCOMP, COLL>, smem);
+    if (e != cudaSuccess) return e;
     dim3 blk(32, 8, 1), grd(p.nx / 32, (p.yhi - p.ylo) / 8, (p.nz + zs - 1) / zs);
     k_lattice_zm<PT, NCOMP, COLL><<<grd, blk, smem, s>>>(*tm, b, p, zs, rev);
     return cudaGetLastError();

@@ -249,13 +249,13 @@ __global__ void __launch_bounds__(kSmallMaxThreads) k_small(StepBufs b, StepPara
     }
 }
 
-// Blocks of the cluster, or 0 where the device takes no cluster of this kernel.
+// Prepares the kernel on the current device; whether it takes the cluster there.
 template <class K>
-int small_cluster(K kernel, int smem_max) {
+bool small_cluster(K kernel, int smem_max) {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_max) != cudaSuccess ||
         cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return false;
     }
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];
@@ -270,16 +270,23 @@ int small_cluster(K kernel, int smem_max) {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        return 0;
+        return false;
     }
-    return n > 0 ? kSmallBlocks : 0;
+    return n > 0;
 }
 
 template <class PT, int NCOMP, int COLL, bool FD>
 cudaError_t small_steps(const StepParams& p, const StepBufs& b, int nsteps, cudaStream_t s) {
     constexpr int node_bytes = SmallPlanes<NCOMP>::total * (int)sizeof(float);
-    static const int blocks = small_cluster(k_small<PT, NCOMP, COLL, FD>, node_bytes * kSmallMaxThreads);
-    if (!blocks) return cudaErrorNotSupported;
+    constexpr int blocks = kSmallBlocks;
+    static PerDevice site;
+    int takes = 0;  // 1 the device takes the cluster, 2 it does not
+    const cudaError_t e = site.get(&takes, [&](int* v) {
+        *v = small_cluster(k_small<PT, NCOMP, COLL, FD>, node_bytes * kSmallMaxThreads) ? 1 : 2;
+        return cudaSuccess;
+    });
+    if (e != cudaSuccess) return e;
+    if (takes != 1) return cudaErrorNotSupported;
     const int m = (((int)p.N + blocks - 1) / blocks + 31) / 32 * 32;
     if (m > kSmallMaxThreads) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};

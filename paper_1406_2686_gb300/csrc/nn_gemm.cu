@@ -26,6 +26,7 @@
 #include <stdint.h>
 
 #include "nn_tc.cuh"
+#include "per_device.cuh"
 #include "vefd_nn.h"
 
 namespace vefd_nn {
@@ -441,13 +442,9 @@ template <int BN>
 cudaError_t launch_tma_bn(const CUtensorMap& ta, const CUtensorMap& tb, float* C, int ldc, int M, int N, int K,
                           int accumulate, int k_split, long long c_split_stride, unsigned* status, cudaStream_t s) {
     constexpr int smem = kStages * (kBM * kBK * 2 + BN * kBK * 2) + 1024;  // + alignment slack
-    static bool attr_set = false;
-    if (!attr_set) {
-        const cudaError_t e =
-            cudaFuncSetAttribute(k_gemm_tma<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static vefd::PerDevice site;
+    const cudaError_t e = vefd::allow_smem(site, k_gemm_tma<BN>, smem);
+    if (e != cudaSuccess) return e;
     static int sms = 0;
     if (!sms) {
         int dev = 0;

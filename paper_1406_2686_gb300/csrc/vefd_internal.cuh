@@ -24,6 +24,8 @@
 #include <utility>
 #include <stdint.h>
 
+#include "per_device.cuh"
+
 namespace vefd {
 
 constexpr float kCs2 = 1.0f / 3.0f;
