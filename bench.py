@@ -142,7 +142,7 @@ def source_hash():
 
 # the translation units and headers the two step kernels (and their launch
 # shapes) are built from
-STEP_KERNEL_SOURCES = ("vefd_internal.cuh", "lbm_impl.cuh", "lbm_kernels.cu", "fd_impl.cuh", "fd_kernels.cu")
+STEP_KERNEL_SOURCES = ("vefd_internal.cuh", "per_device.cuh", "lbm_impl.cuh", "lbm_kernels.cu", "fd_impl.cuh", "fd_kernels.cu")
 
 
 def kernel_source_hash():
