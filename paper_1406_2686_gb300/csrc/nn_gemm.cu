@@ -75,10 +75,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const unsigned bar_a = smem_addr(&bar);
     if (threadIdx.x == 0) mbar_init1(bar_a);
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tmem_alloc(&tmem_base, kTmemCols);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -123,15 +120,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int c0 = 0; c0 < BN; c0 += 16) {
             uint32_t v[16];
             const unsigned taddr = tmem + ((unsigned)(warp * 32) << 16) + (unsigned)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-                "%13, %14, %15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                  "=r"(v[15])
-                : "r"(taddr)
-                : "memory");
-            asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            tmem_ld16(taddr, v);
             if (row < M) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) {
@@ -150,8 +139,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    if (warp == 0) tmem_free(tmem, kTmemCols);
 }
 
 constexpr int kStages = 4;
@@ -224,10 +212,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
         abort_flag = 0;
     }
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_base)),
-                     "r"(kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+        tmem_alloc(&tmem_base, kTmemCols);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -344,15 +329,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
             const unsigned tbase = tmem + ((unsigned)(q * 32) << 16) + (unsigned)acc * kAccCols;
             for (int c0 = 0; c0 < BN; c0 += 16) {
                 uint32_t v[16];
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
-                    "%13, %14, %15}, [%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                      "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]),
-                      "=r"(v[15])
-                    : "r"(tbase + (unsigned)c0)
-                    : "memory");
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+                tmem_ld16(tbase + (unsigned)c0, v);
                 if (row < M) {
                     float* c = Ct + (size_t)row * ldc + n0 + c0;
                     if (n0 + c0 + 16 <= N && !accumulate && ((reinterpret_cast<uintptr_t>(c) & 15u) == 0)) {
@@ -380,8 +357,7 @@ __global__ void __launch_bounds__(kPersistThreads, 1)
     if (failed && lane == 0) atomicOr(status, kStatusTimeout);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    if (warp == 0) tmem_free(tmem, kTmemCols);
 }
 
 }  // namespace

@@ -111,18 +111,23 @@ __device__ __forceinline__ void mma_commit_warp(unsigned bar) {
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
+// The three below are called by a whole warp; .sync.aligned wants it converged,
+// which lanes that left a branch or a loop turn before it need not be.
 __device__ __forceinline__ void tmem_alloc(void* smem_slot, unsigned cols) {
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(smem_slot)), "r"(cols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tmem_free(unsigned base, unsigned cols) {
+    __syncwarp();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(cols) : "memory");
 }
 
 // 16 accumulator columns of this warp's 32 lanes (waits for the load).
 __device__ __forceinline__ void tmem_ld16(unsigned addr, uint32_t v[16]) {
+    __syncwarp();
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, "
         "%13, %14, %15}, [%16];"
@@ -133,7 +138,7 @@ __device__ __forceinline__ void tmem_ld16(unsigned addr, uint32_t v[16]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
-// Tiled bulk tensor copy of one 5-D box into shared memory (128-byte aligned), zero beyond the tensor.
+// Tiled bulk tensor copies of one box into shared memory (128-byte aligned), zero beyond the tensor.
 __device__ __forceinline__ void tma_load_2d(unsigned dst, const CUtensorMap* tm, int c0, int c1, unsigned bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),

@@ -244,3 +244,57 @@ def test_unet_gradients_match_torch(channels):
             assert cos > 0.995 and abs(float(torch.linalg.norm(a) / torch.linalg.norm(r)) - 1) < 0.05, (l.cout, cos)
             assert _rel(a, r) < 0.1
     assert net.status() == 0
+
+
+def _conv_fp64(x, w, dy, stride):
+    """y, dx, dw of a convolution in FP64 tap by tap: x [B][D][H][W][C], w
+    [Cout][27][C], dy as y."""
+    import torch
+    xp = torch.nn.functional.pad(x, (0, 0, 1, 1, 1, 1, 1, 1))
+    B, Do, Ho, Wo, O = dy.shape
+    y, dw, dxp = torch.zeros_like(dy), torch.zeros_like(w), torch.zeros_like(xp)
+    for t in range(27):
+        at = (slice(None), *(slice(o, o + stride * (n - 1) + 1, stride) for o, n in
+                             zip((t // 9, t // 3 % 3, t % 3), (Do, Ho, Wo))))
+        y += xp[at] @ w[:, t].T
+        dw[:, t] = dy.reshape(-1, O).T @ xp[at].reshape(-1, x.shape[-1])
+        dxp[at] += dy @ w[:, t]
+    return y, dxp[:, 1:-1, 1:-1, 1:-1], dw
+
+
+# what the plan for 152 SMs takes each shape through: k_conv's 128-row products
+# and their epilogue with rows beyond the grid, 1, 2 and 4 planes a tile, two to
+# three items a block over two and over one halo buffer and over two and one
+# accumulator sets, and 3 to 18 tiles a block in k_conv_dw's ring of 2 to 4
+@pytest.mark.parametrize("cin,cout,stride,shape", [
+    (16, 16, 1, (1, 61, 58, 64)),   # 4 planes
+    (8, 16, 1, (1, 66, 58, 60)),    # 4 planes, odd slabs
+    (48, 16, 1, (1, 41, 52, 40)),   # 2 planes, three items
+    (112, 32, 1, (1, 36, 44, 60)),  # 2 planes, one halo buffer; gradient of 112 columns
+    (112, 32, 1, (1, 35, 40, 44)),  # 4 planes, one halo buffer; gradient on one accumulator set
+    (40, 24, 2, (1, 60, 44, 72)),   # odd slabs; adjoint on one accumulator set; ring of 2
+    (16, 32, 2, (1, 92, 84, 92)),   # 4 planes of 8 rows
+    (32, 16, 2, (2, 66, 64, 60)),   # two grids
+    (232, 80, 1, (1, 18, 28, 36)),  # 98 weight chunks an item; gradient in three column tiles of 4 planes
+])
+def test_conv_products_over_many_tiles(cin, cout, stride, shape):
+    """The products where a block walks several tiles, against FP64 of the BF16
+    operands; the bound is that of test_conv_products."""
+    import torch
+    from paper_1406_2686_gb300 import nn
+    g = torch.Generator().manual_seed(cin + 3 * cout + stride)
+    lay = nn.Conv3d(cin, cout, stride, False, gen=g)
+    x = torch.randn(*shape, cin, generator=g).cuda()
+    xb = torch.empty(x[..., 0].numel(), nn.round8(cin), dtype=torch.bfloat16, device="cuda")
+    yb = torch.full(lay.out_shape(x.shape), float("nan"), dtype=torch.bfloat16, device="cuda")
+    y = lay._forward(x, xb, x.shape, yb, nn._stream())
+    assert torch.equal(yb, y.to(torch.bfloat16))  # the copy that the next layer reads
+    dy = torch.randn(*y.shape, generator=g).to(torch.bfloat16).float().cuda()
+    dx = lay.backward(dy)
+    assert int(lay.status.item()) == 0
+    w = lay.w.to(torch.bfloat16).double().view(cout, 27, cin)
+    yr, dxr, dwr = _conv_fp64(x.to(torch.bfloat16).double(), w, dy.double(), stride)
+    V = y.numel() // cout
+    for got, ref, K in ((y, yr, 27 * cin), (dx, dxr, 27 * cout), (lay.dw.view(cout, 27, cin), dwr, V),
+                        (lay.db, dy.double().sum((0, 1, 2, 3)), V)):
+        assert float((got.double() - ref).abs().max()) < _tol(ref, K)
