@@ -21,8 +21,11 @@
 //              the eight parities of the input voxels are eight accumulators
 //              over the same staged gradient, each with its one to eight taps).
 //   k_conv_dw  dW^T[(tap, channel)][o] = sum over voxels, one accumulator per tap.
-// Sums over K run tap by tap, 16 channels at a time, in the order of the
-// im2col product (the prediction's bits are those of that product).
+// Sums over K run channel block by channel block (channel_blocks: one block up
+// to 256 channels at stride 1 and 96 at stride 2), in it tap by tap and 16
+// values at a time.  With one block of a multiple of 8 channels that is the
+// order of the im2col product, and the bits are its bits; channels padded to a
+// multiple of 8 and several blocks group the terms differently.
 //
 // Measured, 64^3 unless said: the prediction 330 us (explicit im2col matrices and
 // their scalar kernels: 12263); 48 -> 16 channels forward and backward 171 us

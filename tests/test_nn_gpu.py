@@ -298,3 +298,74 @@ def test_conv_products_over_many_tiles(cin, cout, stride, shape):
     for got, ref, K in ((y, yr, 27 * cin), (dx, dxr, 27 * cout), (lay.dw.view(cout, 27, cin), dwr, V),
                         (lay.db, dy.double().sum((0, 1, 2, 3)), V)):
         assert float((got.double() - ref).abs().max()) < _tol(ref, K)
+
+
+@pytest.mark.parametrize("cin,cout,stride,shape,bits", [
+    (16, 16, 1, (1, 66, 60, 44), True), (24, 16, 1, (1, 20, 18, 24), True), (232, 80, 1, (1, 8, 8, 8), True),
+    (40, 24, 2, (2, 9, 12, 16), True), (256, 32, 1, (1, 4, 8, 8), True), (96, 16, 2, (1, 8, 8, 16), True),
+    (12, 16, 1, (1, 8, 8, 16), False), (264, 16, 1, (1, 4, 8, 8), False), (104, 16, 2, (1, 8, 8, 16), False)])
+def test_conv_layer_agrees_with_the_im2col_route(cin, cout, stride, shape, bits):
+    """The layer against the exported im2col matrices, GEMMs and element kernels.
+    The forward bits are the same where both sum in the same order (one block
+    of a multiple of 8 channels); what is left is FP32 accumulation on both
+    sides, twice the bound of one."""
+    import torch
+    from paper_1406_2686_gb300 import nn
+    g = torch.Generator().manual_seed(cin + cout)
+    lay = nn.Conv3d(cin, cout, stride, True, gen=g)
+    lay.b.copy_(torch.randn(cout, generator=g).cuda() * 0.1)
+    x = torch.randn(*shape, cin, generator=g).cuda()
+    y = lay.forward(x)
+    V, K27, Kp = y.numel() // cout, 27 * cin, nn.round8(27 * cin)
+    dy = torch.randn(*y.shape, generator=g).cuda()
+    lb, s, st = nn.L(), nn._stream(), torch.zeros(1, dtype=torch.int32, device="cuda")
+
+    def empty(*size, dtype=torch.bfloat16):
+        return torch.empty(*size, dtype=dtype, device="cuda")
+
+    def call(name, *args):
+        nn._check(getattr(lb, "vefd_nn_" + name)(*[nn._p(a) if torch.is_tensor(a) else a for a in args], s), name)
+
+    col, colT, wb, wbT = empty(V, Kp), empty(Kp, V), empty(cout, Kp), empty(Kp, cout)
+    call("im2col3d", x, *shape, cin, stride, Kp, col, colT)
+    call("pack_weights", lay.w, cout, K27, Kp, wb, wbT)
+    r = nn.gemm(col, wb, status=st)
+    call("bias_act", r, lay.b, V, cout, 1)
+    r = r.view(y.shape)
+    if bits:
+        assert torch.equal(y, r)
+    assert float((y - r).abs().max()) < 2 * _tol(r, K27)
+
+    # the gradients for one forward output: the mask is then the same
+    lay._saved = (x.shape, lay._saved[1], r)
+    dx = lay.backward(dy)
+    f32 = torch.float32
+    gr, gb, gbT = empty(V, cout, dtype=f32), empty(V, cout), empty(cout, V)
+    call("act_backward", dy, r, V, cout, 1, gr, gb, gbT)
+    db, dw = empty(cout, dtype=f32), empty(cout, K27, dtype=f32)
+    call("colsum", gr, V, cout, empty(lb.vefd_nn_colsum_scratch(V, cout), dtype=f32), db, 0)
+    ks = 64 * ((V + 255) // 256)
+    splits = (V + ks - 1) // ks
+    parts = empty(splits, Kp, cout, dtype=f32)
+    nn._check(lb.vefd_nn_gemm_bf16_splitk(colT.data_ptr(), V, gbT.data_ptr(), V, parts.data_ptr(), cout, Kp, cout, V, ks,
+                                          Kp * cout, st.data_ptr(), s), "splitk")
+    call("splitk_reduce_t", parts, splits, Kp * cout, Kp, cout, K27, dw, 0)
+    dcol, dxr = nn.gemm(gb, wbT, status=st), empty(*x.shape, dtype=f32)
+    call("col2im3d", dcol, *shape, cin, stride, Kp, dxr)
+    assert int(st.item()) == 0 and int(lay.status.item()) == 0
+    for a, b, K in ((dx, dxr, 27 * cout), (lay.dw, dw, V), (lay.db, db, V)):
+        assert float((a - b).abs().max()) < 2 * _tol(b, K)
+
+
+def test_upsample_and_concat():
+    """The FP32 forms of what the network's fused pass does: copies, so exact."""
+    import torch
+    from paper_1406_2686_gb300 import nn
+    g = torch.Generator().manual_seed(2)
+    u, sk = (torch.randn(2, d, d + 1, d + 2, c, generator=g).cuda() for d, c in ((3, 16), (3, 8)))
+    up = nn.upsample2(u)
+    for k in (1, 2, 3):
+        u = u.repeat_interleave(2, dim=k)
+        sk = sk.repeat_interleave(2, dim=k)
+    assert torch.equal(up, u)
+    assert torch.equal(nn.concat(up, sk.contiguous()), torch.cat([u, sk], dim=-1))
