@@ -249,9 +249,7 @@ vefd_status vefd_kernel_times(vefd_ctx *ctx, double ms[3], int64_t launches[3]);
  * (about 3 values per node) instead of reading the new populations back; the
  * partial sums use the staging planes, which are free inside a step.  Post
  * modes 1 and 2 with tiles 0-2 run the same arithmetic in the
- * same order and give bit-identical results (with the FP32 moment-space
- * collision on lattices the column does not fit, tile 0 agrees with tiles 1
- * and 2 to FP32 rounding); the persistent tiles (separately
+ * same order and give bit-identical results; the persistent tiles (separately
  * compiled, multiply-adds contracted as the compiler sees fit) and post modes 0
  * and 3 (each node's new density summed in another order) agree to FP32
  * rounding.  A tile the lattice shape

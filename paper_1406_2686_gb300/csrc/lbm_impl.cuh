@@ -278,6 +278,13 @@ __device__ __forceinline__ void pi_add(float pi[6], int a, float fa) {
     if (cz) pi[5] += fa;
 }
 
+// f + sign * wall for sign -1, 0 or 1, where wall is a rounded product: left to
+// the compiler, product and sum were contracted in some instantiations and not
+// in others, and the bits of a lattice with moving walls depended on its route.
+__device__ __forceinline__ float add_wall(float f, int sign, float wall) {
+    return sign > 0 ? __fadd_rn(f, wall) : sign < 0 ? __fsub_rn(f, wall) : f;
+}
+
 // Collision of every population of every component and push streaming.
 // fget(s, a) returns the stored deviation f_a^s of this node; pif[s] the
 // second moments of component s's stored deviations (moment-space collision).
@@ -416,7 +423,7 @@ __device__ __forceinline__ void collide_emit(const StepParams& p, const Local<NC
             const float k0 = wa * K0;
             const float rx = wa * Rx, ry = wa * Ry, rz = wa * Rz;
             const float px = wa * Px, py = wa * Py, pz = wa * Pz;
-            const float wrs = wa * rsv, tqw = wa * tqo;
+            const float wall = __fmul_rn(wa * rsv, uw6), tqw = wa * tqo;
 #pragma unroll
             for (int a = 1; a < L::Q; a += 2) {
                 if ((L::w(a) == w_axis) != (wc == 0)) continue;
@@ -451,9 +458,9 @@ __device__ __forceinline__ void collide_emit(const StepParams& p, const Local<NC
                 // the moving-wall term -2 w rho_s (c.U)/c_s^2 (+U lower, -U upper)
                 const bool ba = (cy > 0 && wall_hi) || (cy < 0 && wall_lo);
                 const bool bb = (cy < 0 && wall_hi) || (cy > 0 && wall_lo);
-                const PT va = pop_put<PT>(ba ? fa - wrs * (float)cx * (cy < 0 ? uw6 : -uw6) : fa);
+                const PT va = pop_put<PT>(ba ? add_wall(fa, cy < 0 ? -cx : cx, wall) : fa);
                 moved += pop_get(va);
-                const PT vb = pop_put<PT>(bb ? fb + wrs * (float)cx * (cy > 0 ? uw6 : -uw6) : fb);
+                const PT vb = pop_put<PT>(bb ? add_wall(fb, cy > 0 ? cx : -cx, wall) : fb);
                 moved += pop_get(vb);
                 emit(s, a, va, vb, ba, bb);
             }
@@ -595,9 +602,7 @@ __device__ __forceinline__ void node_collide(const StepBufs& b, const StepParams
 // that 168 registers allow, and 4 and 6: 100 x 50 x 70 27.4 us (4: 29.7, 6:
 // 29.3).  The FP32 moment-space collision, which reads its populations twice
 // (see k_lattice), takes 6: the same box 25.1 us (5: 26.3, 7: 26.3).  16-bit
-// storage takes 4 (24.7 us, 5: 24.2, 3: 26.7): at 96 registers the compiler
-// rounds the moving-wall term in another order than in the staged kernels, which
-// 16-bit storage turns into flipped last bits.
+// storage takes 4 (24.7 us, 5: 24.2, 3: 26.7); the count changes no bit.
 template <class PT, class L, int COLL>
 constexpr int reg_blocks() {
     return sizeof(PT) == 2 ? 4 : L::D == 3 && COLL == 1 ? 6 : 5;

@@ -372,9 +372,9 @@ uint64_t splitmix64(uint64_t seed, uint64_t i) {
 //   14.4 against 13.6.
 // - D3Q19, moment-space collision: 16-bit storage always (256 x 128 x 64 108
 //   against 112 us, 116 x 50 x 70 26.7 and 27.1), FP32 where the z-marching column
-//   fits: runs are faster (64^3 20.7 us in boxes, 19.7 in runs; 132 x 70 x 100 73.2
-//   and 59.8) but may round the moving-wall term differently, and lattices that
-//   the slab graph and the ensembles take give the same bits on every route.
+//   fits, as the slab graph and the ensembles (64^3 20.7 us in boxes, 19.7 in runs),
+//   and runs elsewhere (132 x 70 x 100 73.2 us in boxes, 59.8 in runs).
+// The bits are the same either way.
 bool lattice_boxes(const vefd_ctx* c) {
     if (!c->tma_ok) return false;
     if (c->lat_tile != 0 || c->parts_ok) return true;

@@ -88,3 +88,38 @@ def test_many_steps_in_one_launch_give_the_bits_of_single_steps(box, collision):
     for f in (vefd.POPS, vefd.C, vefd.RPREV, vefd.U, vefd.PHI, vefd.RHO_A):
         a, b = A.read(f), B.read(f)
         assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("flow", ["walls", "walls_force", "periodic_force"])
+@pytest.mark.parametrize("precision", [0, 1, 2])
+@pytest.mark.parametrize("ncomp", [1, 2])
+@pytest.mark.parametrize("collision", [0, 1])
+@pytest.mark.parametrize("lattice", [0, 1])
+def test_routes_leave_the_same_bits(lattice, collision, ncomp, precision, flow, monkeypatch):
+    """Runs, staged boxes of two shapes, the unstaged kernels, the whole-lattice
+    graph and (D2Q9) many steps in one launch, with moving walls, a body force
+    and each storage type: no bit depends on the route."""
+    from paper_1406_2686_gb300 import vefd
+    box = dict(COMMON, lattice=lattice, ncomp=ncomp, precision=precision)
+    box.update(dict(nx=48, ny=35) if lattice == 0 else dict(nx=40, ny=9, nz=7))  # the default takes runs, except 16-bit moment space
+    walls = int(flow != "periodic_force")
+    box.update(walls=walls, u_wall=0.03 * walls, fext=(1e-5, 2e-5, -1e-5) if "force" in flow else (0.0, 0.0, 0.0))
+    if ncomp == 1:
+        box.update(G=0.0, phase=0)
+
+    def run(config=None, graph=0):
+        L = make(box, seed=9)
+        if config:
+            L.set_kernel_config(*config)
+        L.set_step_graph(graph)
+        L.set_collision(collision)
+        L.step(6)
+        return state(L) + (L.read(vefd.U),)
+
+    ref = run((1, 1))
+    others = {"runs": run(), "box 2": run((2, 1)), "graph": run(graph=1), "automatic": run(graph=-1)}
+    monkeypatch.setenv("VEFD_NO_TMA", "1")
+    others["unstaged"] = run()
+    assert all(np.isfinite(a).all() for a in ref)
+    for name, got in others.items():
+        assert all(np.array_equal(a, b) for a, b in zip(got, ref)), name
