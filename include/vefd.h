@@ -269,8 +269,8 @@ vefd_status vefd_set_kernel_config(vefd_ctx *ctx, int lattice_tile, int post_mod
  *   VEFD_SCHEDULE=b      bit 0 walks the lattice kernel's tiles, bit 1 the pass's
  *                        columns in reverse order (default 0);
  *   VEFD_ZM_SEGMENT=n    z-segment length of the column march (default: one wave);
- *   VEFD_SLAB_SEGMENT=n  z-segment of the step graph's slab passes (default: 12 to 64
- *                        planes, so that a slab has 64 blocks);
+ *   VEFD_SLAB_SEGMENT=n  z-segment of the step graph's slab passes (default: as long as
+ *                        a slab has 64 blocks, but 12 planes at least, 64 at most);
  *   VEFD_SLAB_PDL=1      programmatic launch between a slab's consecutive kernels
  *                        inside the step graph (measured slower; off). */
 /* The configuration in effect: lattice_tile -1 and post_mode -1 mean the
@@ -304,8 +304,8 @@ vefd_status vefd_autotune(vefd_ctx *ctx, int steps, double *times_ms);
  *   of step n on slabs k-1, k, k+1, and its pass of step n waits for the
  *   lattice kernels of step n on those slabs.  Work on different slabs then
  *   overlaps, and a slab's new populations can be re-read while still in L2.
- *   Each slab's pass marches z-segments of 12 to 64 planes, as long as they
- *   leave the slab 64 blocks.  This form needs: D3Q19; a staged tile 0-2 with post mode 2;
+ *   Each slab's pass marches z-segments that leave the slab 64 blocks, but
+ *   of 12 planes at least and 64 at most.  This form needs: D3Q19; a staged tile 0-2 with post mode 2;
  *   NY a multiple of 8 * slabs.  An explicit slab count the lattice does not
  *   admit means eager stepping.
  * - Whole-lattice (slabs = 1): the eager launch pairs of `chunk` steps,

@@ -429,7 +429,7 @@ int slab_count(const vefd_ctx* c) {
 }
 
 // z-segment of the pass on one of K slabs: as long as the slab still gives 64
-// blocks, from 12 to 64 planes.  A segment reads two planes beyond its own, so
+// blocks, but 12 planes at least (44 blocks on 128 x 64 x 128) and 64 at most.  A segment reads two planes beyond its own, so
 // long ones move fewer bytes; too few blocks leave the SMs waiting for a slab.
 // Steps in us with 12 / 16 / 32 / 64 planes: 128 x 64 x 128 (4 columns a slab) 106 /
 // 113 / 139 / 207, 192 x 64 x 192 (6) 240 / 236 / 244 / 299, 128^3 (8) 208 / 205 / 218 /
@@ -1840,9 +1840,10 @@ void ens_sets(const vefd_ensemble* e, std::vector<int>* order, std::vector<int>*
 
 // Whether the automatic form is that of branches although the members admit
 // batched launches: their mean size is 2^14 to 2^19 nodes and no z-segment, group
-// count or tile 1 was set.  Smaller
-// ones are bound by their launches (64 of 32 x 16 x 16: 61 us batched, 49 in sets, but
-// four times the graph), larger ones gain nothing (2 of 128 x 64 x 128 217 / 219).
+// count or tile 1 was set.  Larger ones gain nothing (2 of 128 x 64 x 128 217 / 219).
+// Smaller ones step faster in branches too (us a step batched / in branches: 64 of
+// 32 x 16 x 16 61 / 49, 256 of them 233 / 184) but keep the batched form, whose graph
+// has eight launches a step however many members there are.
 bool ens_prefers_sets(const vefd_ensemble* e) {
     long long total = 0;
     for (const vefd_ctx* m : e->members) total += m->N;

@@ -144,16 +144,6 @@ __device__ __forceinline__ float pop_again(const float* p) {
     asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ float pop_again(const __half* p) {
-    unsigned short v;
-    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return __half2float(__ushort_as_half(v));
-}
-__device__ __forceinline__ float pop_again(const __nv_bfloat16* p) {
-    unsigned short v;
-    asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
-    return __bfloat162float(__ushort_as_bfloat16(v));
-}
 
 // volatile shared-memory read of a staged population (keeps it out of registers)
 __device__ __forceinline__ float pop_smem(const float* base, int idx) {
