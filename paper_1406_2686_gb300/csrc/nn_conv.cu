@@ -33,8 +33,11 @@
 // conversion, mask and sums; 232 -> 80 at 16^3 101 us (780).  Deep levels are one
 // chain a tile: at 16^3 392 steps on one accumulator at 85 clocks, beside which
 // setup (2k clocks), the halo's 9000 pieces (10k), and 49 chunks of weights count;
-// the fine levels are bound by the tensor core's 39 clocks a step of 16 columns
-// (22 us of the 43) and the staging of 16-byte pieces.  What made the chain
+// 48 -> 16 at 64^3 by the tensor core's 39 clocks a step of 16 columns (22 us of
+// the 43) and the staging of 16-byte pieces.  The layers of 8 and 16 channels at
+// 64^3 take 22-24 us each, of which the tensor core needs 4 to 7: one or two items a
+// block, so set-up, staging, steps and the epilogue's FP32 and BF16 stores (17 and 8
+// MB) follow one another more than they overlap.  What made the chain
 // shorter: weights of part of the columns by one box a chunk instead of 2 x chunk
 // small copies (forward at 16^3 49.0 to 42.2 us together with halo planes that
 // land in three groups), and waits of one poll (prediction 345 to 330 us).

@@ -1842,8 +1842,9 @@ void ens_sets(const vefd_ensemble* e, std::vector<int>* order, std::vector<int>*
 // batched launches: their mean size is 2^14 to 2^19 nodes and no z-segment, group
 // count or tile 1 was set.  Larger ones gain nothing (2 of 128 x 64 x 128 217 / 219).
 // Smaller ones step faster in branches too (us a step batched / in branches: 64 of
-// 32 x 16 x 16 61 / 49, 256 of them 233 / 184) but keep the batched form, whose graph
-// has eight launches a step however many members there are.
+// 32 x 16 x 16 61 / 49, 256 of them 230 / 179) but keep the batched form, whose graph
+// has eight launches a step however many members there are: the first 32 steps
+// of the 256 take 8.3 ms with their capture, in branches 49 ms.
 bool ens_prefers_sets(const vefd_ensemble* e) {
     long long total = 0;
     for (const vefd_ctx* m : e->members) total += m->N;
